@@ -507,6 +507,7 @@ int factor_direction(ls_handle* h, int dir, Scratch& S) {
     LS_CUDA(cudaMemcpyAsync(&herr, S.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     LS_CUDA(cudaStreamSynchronize(h->stream));
     if (herr) return LS_ESINGULAR;
+    LS_TRY(ls_cr_inverse_build(h, dir));
     if (h->prec == LS_MIXED) {
         const size_t cnt = qq * F.mats_per_strip * L;
         LS_CUDA(cudaMalloc(&F.pool32, sizeof(float2) * cnt));
@@ -537,6 +538,8 @@ void ls_factor_free(ls_handle* h) {
         cudaFree(F.cw);
         cudaFree(F.ce);
         cudaFree(F.cinj);
+        cudaFree(F.inv);
+        F.inv = nullptr;
         F.pool64 = nullptr;
         F.pool32 = nullptr;
         F.cw = F.ce = F.cinj = nullptr;

@@ -176,6 +176,10 @@ struct DirFactors {
     // levels >= dense_c of a local solve are one dense product (ls_cr_dense_apply)
     float* dense_tc = nullptr;
     int dense_c = 0, dense_nc = 0, dense_mt = 0, dense_ks = 0;
+    // CUDA-core steps: the inverse of the reduced system of level inv_c, inv_nc unknowns,
+    // column-major per strip, in the solves' precision (ls_cr_inverse_build)
+    void* inv = nullptr;
+    int inv_c = 0, inv_nc = 0;
     // problem of this direction (the vertical direction is the transposed grid)
     const double* m = nullptr;    // medium of this direction's grid (n x n, long axis fastest)
     StencilTables* tab = nullptr; // device copy of the tables of this direction
@@ -245,8 +249,7 @@ struct ls_handle {
         cudaGraphExec_t exec[kMaxBatch + 1] = {};
         long long nodes[kMaxBatch + 1] = {};
         int nb_cap = 0;
-        void* cr_part = nullptr;        // partial sums of split reduction steps
-        unsigned* cr_cnt = nullptr;     // arrival counters of split reduction steps (kept at 0)
+        void* cr_y = nullptr;           // y_j of a local solve's odd blocks (CUDA-core steps): n * q each
         float2* dense_part = nullptr;   // column-chunk partial products of the reduced inverse
         cudaStream_t stream = nullptr;  // lane 0 runs on the handle's stream
         cudaEvent_t done = nullptr;
@@ -316,6 +319,34 @@ int ls_cuda_fail(cudaError_t e);
         cudaError_t e_ = cudaPeekAtLastError();                                        \
         if (e_ != cudaSuccess) return ls_cuda_fail(e_);                                \
     } while (0)
+
+// Programmatic dependent launch: a kernel launched this way may start while its predecessor
+// on the stream still runs, once every CTA of the predecessor has called pdl_trigger (or
+// ended).  Until its own pdl_wait -- which returns when the predecessor has completed and its
+// writes are visible -- it may touch only data that no kernel still in flight writes (the
+// factors and tables of ls_factor).  Every kernel of such a chain calls pdl_wait, so a
+// completed predecessor implies that everything before it has completed too.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+int ls_launch_pdl(ls_handle* h, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+    h->launches++;
+    return e == cudaSuccess ? LS_OK : ls_cuda_fail(e);
+}
+#endif
 
 // ------------------------------------------------------------------ internal API
 // FFT convolution (ls_fft.cu)
@@ -390,6 +421,7 @@ int ls_bd(ls_handle* h, const double2* g, double2* v);                   // Algo
 int ls_bd_cap(const ls_handle* h);   // right-hand sides one Algorithm 2 pass takes: FP64 4, mixed 8 (32 on tensor cores)
 void ls_bd_graph_free(ls_handle* h);
 int ls_strip_solve(ls_handle* h, int dir, int layer, const double2* b, double2* x);
+int ls_cr_inverse_build(ls_handle* h, int dir);   // from the complete FP64 factors (ls_factor)
 
 // tensor-core reduction steps (ls_cr_mma.cu)
 int ls_cr_tc_prepare(ls_handle* h);

@@ -24,13 +24,11 @@
 //
 // Local solve (C^l)^{-1} b by the block cyclic reduction factors of ls_factor.cu:
 //   forward  level 0:  y_j = D_j^{-1} b_j (odd j);  b_j -= W_j y_{j-1} + E_j y_{j+1} (even j)
-//            level k:  b_j -= F_j b_{j-1} + G_j b_{j+1} (even j of level k)
-//   top:     x_0 = D^{-1} b_0
-//   backward level k:  x_j = D_j^{-1} b_j - P_j x_{j-1} - Q_j x_{j+1} (odd j)
+//            level k:  b_j -= F_j b_{j-1} + G_j b_{j+1} (even j of level k),  y_j = D_j^{-1} b_j (odd j)
+//   level c: x = S_c^{-1} b (the reduced system's precomputed inverse)
+//   backward level k:  x_j = y_j - P_j x_{j-1} - Q_j x_{j+1} (odd j)
 //            level 0:  x_j = y_j - D_j^{-1} (W_j x_{j-1} + E_j x_{j+1}) (odd j)
-// Each kernel is one launch per level over all blocks of that level; a block of
-// 256 threads handles one block's mat-vecs, its warps splitting the columns of
-// the column-major matrices (coalesced reads, all loads independent).
+// Each kernel is one launch per level over all blocks of that level.
 //
 // Batches: every kernel takes nb right-hand sides at once (batch member b's
 // strips at offset b * SB, its grid vectors at offset b * N).  A reduction step
@@ -43,215 +41,381 @@
 
 namespace {
 
+constexpr int kMvThreads = 256;
+
+// Right-hand side of a local solve, block i (a strip column), row r, member b: the gathered
+// field plus the injections of Algorithm 1, formed where level 0 reads it, so that the chain
+// of a sweep holds no kernels but the reduction steps.  Rows E+t-1 and E+t take the traces of
+// the layer above (its down-sweep solution, which stays in place until the upward sweep has
+// passed this layer), rows E-1 and E those of the layer below (upward sweep only).
 template <typename T>
-struct Pool {
-    const cpx_t<T>* base;  // strip l's first matrix
-    size_t qq;
-    __device__ __forceinline__ const cpx_t<T>* mat(size_t off) const { return base + off * qq; }
+struct RhsSrc {
+    using C = cpx_t<T>;
+    const C* rhs;      // gathered g^l; member b at + b * SB (never written by the solve)
+    const C* inj;      // cinj of layer l: [slot][dx+1][i]
+    const C* above;    // solution of layer l + 1, or null
+    const C* below;    // solution of layer l - 1 (upward sweep), or null
+    const C* tself;    // w^l_0 of the down sweep (upward sweep); member b at + b * TB
+    C* tsave;          // where w^{l+1}_0 is kept for the upward sweep (down sweep), or null
+    size_t SB, TB;
+    int n, q, E, t;
+    __device__ __forceinline__ C load(int i, int r, int b) const {
+        const size_t mo = (size_t)b * SB;
+        C val = rhs[mo + (size_t)i * q + r];
+        if (above) {
+            if (r == E + t - 1) {  // -C^l_{n,n+1} w^{l+1}_1 ; w^{l+1}_1 = row E of layer l+1
+                for (int dx = -1; dx <= 1; ++dx)
+                    if (i + dx >= 0 && i + dx < n)
+                        val = cfms(inj[(size_t)(0 * 3 + dx + 1) * n + i], above[mo + (size_t)(i + dx) * q + E], val);
+            } else if (r == E + t) {  // +C^l_{n+1,n} w^{l+1}_0 ; w^{l+1}_0 = row E-1 of layer l+1
+                for (int dx = -1; dx <= 1; ++dx)
+                    if (i + dx >= 0 && i + dx < n)
+                        val = cfma(inj[(size_t)(1 * 3 + dx + 1) * n + i], above[mo + (size_t)(i + dx) * q + E - 1], val);
+            }
+        }
+        if (below) {
+            if (r == E) {  // -C^l_{1,0} (v^{l-1}_n - w^l_0) ; v^{l-1}_n = row E+t-1 of layer l-1
+                for (int dx = -1; dx <= 1; ++dx) {
+                    if (i + dx < 0 || i + dx >= n) continue;
+                    const C p0 = below[mo + (size_t)(i + dx) * q + E + t - 1] - tself[(size_t)b * TB + i + dx];
+                    val = cfms(inj[(size_t)(2 * 3 + dx + 1) * n + i], p0, val);
+                }
+            } else if (r == E - 1) {  // +C^l_{0,1} v^{l-1}_{n+1} ; v^{l-1}_{n+1} = row E+t of layer l-1
+                for (int dx = -1; dx <= 1; ++dx) {
+                    if (i + dx < 0 || i + dx >= n) continue;
+                    val = cfma(inj[(size_t)(3 * 3 + dx + 1) * n + i], below[mo + (size_t)(i + dx) * q + E + t], val);
+                }
+            }
+        }
+        return val;
+    }
+    __device__ __forceinline__ void keep_trace(int i, int b) const {
+        if (tsave) tsave[(size_t)b * TB + i] = above[(size_t)b * SB + (size_t)i * q + E - 1];
+    }
 };
 
-constexpr int kMvWarps = 8;
-constexpr int kMvThreads = 32 * kMvWarps;
+// The tridiagonal couplings of level 0 (blocks W_i, E_i) of one strip: [i][dz+1][r]
+template <typename T>
+struct Couple {
+    const cpx_t<T>* cw;
+    const cpx_t<T>* ce;
+};
 
-// One reduction step for one block j and NB (>= nb) batch members:
+// One reduction step.  A CTA takes one block j of the level and a chunk of R of its rows (S
+// chunks a block) for NB (>= nb) batch members:
 //   out_b = base_b + sum_t M_t v_{t,b}
-// Warp w takes columns w, w + 8, ...; lane l takes rows l, l + 32, ... (RPT rows);
-// each matrix entry is loaded once and used for every batch member; the
-// vectors (signs applied) sit in shared memory, partial sums are reduced there.
-//   MODE 0 (level 0 odd):    x_j = D^{-1} x_j
-//   MODE 1 (forward):        x_j = x_j - F x_{j-1} - G x_{j+1}          (even j)
-//   MODE 2 (backward):       x_j = D^{-1} x_j - P x_{j-1} - Q x_{j+1}   (odd j)
-//   MODE 3 (top block):      x_0 = D^{-1} x_0
+//   MODE 0 (level 0 odd):     x_j = D^{-1} b_j
+//   MODE 1 (forward, k >= 2): even j: x_j = x_j - F x_{j-1} - G x_{j+1};  odd j: y_j = D^{-1} x_j
+//   MODE 5 (forward, k = 1):  the same with the level-0 even update b'_i = b_i - W_i y_{i-1}
+//          - E_i y_{i+1} formed as the blocks are read (it is never stored)
+//   MODE 2 (backward):        x_j = y_j - P x_{j-1} - Q x_{j+1}   (odd j, levels >= 1)
+//   MODE 3 (top block):       x_0 = D^{-1} x_0   (S = 1; only to build the reduced inverse)
+//   MODE 4 (level 0 back):    x_j = x_j - D^{-1} (W_j x_{j-1} + E_j x_{j+1})   (odd j)
+//   MODE 6 (level c):         x = S_c^{-1} y over all nc unknowns of the level
 //
-// Split levels (S > 1, for levels with fewer blocks than the GPU has SMs): S CTAs
-// share a block, CTA p taking the columns [p q / S, (p+1) q / S) of its matrices.
-// Each writes its partial sums to `partial`, and the CTA that arrives last at the
-// block's counter (an atomic increment; nobody waits) adds the S partials in the
-// fixed order p = 0..S-1, writes the block's result and resets the counter.  The
-// result does not depend on which CTA arrives last, and x_j is overwritten only
-// after every CTA of the block has read it.
-template <typename T, int RPT, int MODE, int NB>
-__global__ void __launch_bounds__(kMvThreads, NB >= 4 ? 2 : 1) k_cr_step(int q, int k, int nk, Pool<T> pool, size_t off_a,
-                                                       size_t off_b, size_t off_c, cpx_t<T>* __restrict__ x,
-                                                       size_t SB, int nb, int S, cpx_t<T>* __restrict__ partial,
-                                                       unsigned* __restrict__ counter) {
+// What bounds a step is latency: a local solve is a chain of dependent steps, most over a few
+// blocks.  On GB300 a chain of trivial kernels takes 1.0 us a link, and handing partial sums
+// from CTA to CTA through global memory adds 2.5 us.  So
+//   * a level with few blocks is split by rows, which needs no sums across CTAs.  No CTA
+//     writes what another one reads: D^{-1} b of the odd blocks is taken on the forward way,
+//     into y, where it is off the backward chain and frees x_j for writing;
+//   * thread (cg, rr) takes row rr of the chunk and columns cg, cg + CG, ... (CG = 256 / R):
+//     no lane idles on rows past q (FP64 runs at 1/64 of the FP32 rate: at q = 70 rows padded
+//     to warps cost 37 per cent), and the CG partial sums meet in shared memory;
+//   * every step is launched programmatically and loads its first PF columns per thread and
+//     its coupling tables (constant data) while its predecessor runs; the register window then
+//     stays PF columns ahead of the products.  A step lets its successor start at once (one
+//     FP32 member: bytes are short), when it has its vectors, or (FP64, few CTAs) at its end:
+//     a successor placed while CTAs still run fills the idle SMs first, two or three CTAs
+//     each, and the FP64 pipe of those then holds everyone up (a 64^2 FP64 solve: 53 us with
+//     the trigger at once, 41 after the vectors, 36 at the end; at 400^2 145, 144 and 154 us,
+//     so steps of more CTAs keep the second form).
+// A local solve of one right-hand side went from 126.6 to 71 us (768^2, FP32), from 219 to
+// 141 us (400^2, FP64: 27 million multiply-adds, 50 us at the FP64 rate) and from 83 to 36 us
+// (64^2, FP64).
+template <typename T>
+struct CrStep {
     using C = cpx_t<T>;
-    constexpr int NM = MODE == 1 ? 2 : (MODE == 2 ? 3 : 1);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int last;
-    C* vin = reinterpret_cast<C*>(smem_raw);     // [NM][NB][q]
-    C* red = vin + (size_t)NM * NB * q;          // [kMvWarps][NB][q]
-    const int idx = blockIdx.x / S, sp = blockIdx.x - idx * S;
-    const int cbeg = q * sp / S, cend = q * (sp + 1) / S;
-    const size_t s = (size_t)1 << k;
-    const int j = MODE == 1 ? 2 * idx : (MODE == 3 ? 0 : 2 * idx + 1);
-    const bool hw = j >= 1, he = j + 1 < nk;
-    for (int o = threadIdx.x; o < NM * NB * q; o += kMvThreads) {
-        const int t = o / (NB * q), b = (o / q) % NB, r = o % q;
-        C val = czero<C>();
-        if (b < nb) {
-            const C* xb = x + (size_t)b * SB;
-            if (MODE == 0 || MODE == 3) val = xb[((size_t)j * s) * q + r];
-            if (MODE == 1) {
-                if (t == 0 && hw) val = -xb[((size_t)(j - 1) * s) * q + r];
-                if (t == 1 && he) val = -xb[((size_t)(j + 1) * s) * q + r];
-            }
-            if (MODE == 2) {
-                if (t == 0) val = xb[((size_t)j * s) * q + r];
-                if (t == 1) val = -xb[((size_t)(j - 1) * s) * q + r];
-                if (t == 2 && he) val = -xb[((size_t)(j + 1) * s) * q + r];
-            }
-        }
-        vin[o] = val;
-    }
-    __syncthreads();
-    const C* Ms[NM];
-    if (MODE == 0 || MODE == 3) Ms[0] = pool.mat(off_a + idx);
-    if (MODE == 1) {  // a missing neighbour has zero vectors; its matrix slot reuses the other one
-        const C* F = pool.mat(off_b + idx);
-        const C* G = pool.mat(off_c + idx);
-        Ms[0] = hw ? F : G;
-        Ms[NM - 1] = he ? G : F;
-    }
-    if (MODE == 2) {
-        const C* Dm = pool.mat(off_a + idx);
-        Ms[0] = Dm;
-        Ms[1] = pool.mat(off_b + idx);
-        Ms[NM - 1] = he ? pool.mat(off_c + idx) : Dm;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    C part[RPT][NB];
-#pragma unroll
-    for (int kk = 0; kk < RPT; ++kk)
-#pragma unroll
-        for (int b = 0; b < NB; ++b) part[kk][b] = czero<C>();
-#pragma unroll 2
-    for (int c = cbeg + warp; c < cend; c += kMvWarps) {
-        C a[NM][RPT];
-#pragma unroll
-        for (int t = 0; t < NM; ++t)
-#pragma unroll
-            for (int kk = 0; kk < RPT; ++kk) {
-                const int r = lane + 32 * kk;
-                a[t][kk] = r < q ? __ldg(&Ms[t][(size_t)c * q + r]) : czero<C>();
-            }
-#pragma unroll
-        for (int t = 0; t < NM; ++t)
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const C vc = vin[((size_t)t * NB + b) * q + c];
-#pragma unroll
-                for (int kk = 0; kk < RPT; ++kk) part[kk][b] = cfma(a[t][kk], vc, part[kk][b]);
-            }
-    }
-#pragma unroll
-    for (int kk = 0; kk < RPT; ++kk) {
-        const int r = lane + 32 * kk;
-        if (r < q)
-#pragma unroll
-            for (int b = 0; b < NB; ++b) red[((size_t)warp * NB + b) * q + r] = part[kk][b];
-    }
-    __syncthreads();
-    if (S == 1) {
-        for (int o = threadIdx.x; o < nb * q; o += kMvThreads) {
-            const int b = o / q, r = o % q;
-            C sum = czero<C>();
-            for (int w = 0; w < kMvWarps; ++w) sum = sum + red[((size_t)w * NB + b) * q + r];
-            C* xj = x + (size_t)b * SB + ((size_t)j * s) * q;
-            xj[r] = MODE == 1 ? xj[r] + sum : sum;
-        }
-        return;
-    }
-    C* mine = partial + ((size_t)idx * S + sp) * NB * q;
-    for (int o = threadIdx.x; o < nb * q; o += kMvThreads) {
-        const int b = o / q, r = o % q;
-        C sum = czero<C>();
-        for (int w = 0; w < kMvWarps; ++w) sum = sum + red[((size_t)w * NB + b) * q + r];
-        mine[(size_t)b * q + r] = sum;
-    }
-    __threadfence();   // the partial is visible before the counter says so
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&counter[idx], 1u) == (unsigned)(S - 1);
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int o = threadIdx.x; o < nb * q; o += kMvThreads) {
-        const int b = o / q, r = o % q;
-        C tot = czero<C>();
-        for (int p = 0; p < S; ++p) tot = tot + __ldcg(&partial[(((size_t)idx * S + p) * NB + b) * q + r]);
-        C* xj = x + (size_t)b * SB + ((size_t)j * s) * q;
-        xj[r] = MODE == 1 ? xj[r] + tot : tot;
-    }
-    if (threadIdx.x == 0) counter[idx] = 0u;
+    int q, k, nk;                  // strip height, level, blocks of the level
+    int S, R;                      // row chunks per block (MODE 6: in all), rows of a chunk
+    int nlead;                     // MODE 1, 5: CTAs on even blocks (the odd blocks' follow)
+    const C* pool;                 // first matrix of the strip (q x q, column-major)
+    size_t off_a, off_b, off_c;    // level offsets (matrices): D^{-1}; F or P; G or Q
+    C* x;                          // strip vectors; member b at + b * SB
+    C* y;                          // y_j of the odd blocks of levels >= 1; at level c, its right-hand side
+    size_t SB, YB;                 // member strides
+    size_t pool_strip, x_strip;    // strip blockIdx.y (elements; the set-up runs all strips at once)
+    int nb;
+    bool to_y;                     // MODE 1, 5: the even results go to y (the last level before c)
+    const C* inv;                  // MODE 6: S_c^{-1} (nc x nc, column-major), blocks j << c
+    int nc, c;
+    RhsSrc<T> src;                 // MODE 0, 5
+    Couple<T> cp;                  // MODE 4, 5
+};
+
+template <int MODE> constexpr int cr_mats() { return MODE == 1 || MODE == 2 || MODE == 5 ? 2 : 1; }   // matrices
+template <int MODE> constexpr int cr_vecs() { return MODE == 5 ? 3 : cr_mats<MODE>(); }                // vectors
+template <int MODE> constexpr int cr_tabs() { return MODE == 5 ? 3 : (MODE == 4 ? 1 : 0); }            // coupling tables
+// columns a thread keeps in flight: 24 (FP64 32) registers of matrix entries, so that (FP32) four CTAs
+// share an SM: 768^2, one member, 71 us a solve against 80 with 40 registers, 78 with five
+// CTAs of 48 and 89 with three of 80
+template <typename T, int MODE> constexpr int cr_prefetch() { return (sizeof(T) == 8 ? 8 : 12) / cr_mats<MODE>() - (MODE == 5 ? 1 : 0); }
+template <typename T, int NB> constexpr int cr_min_ctas() { return sizeof(T) == 8 ? (NB <= 2 ? 3 : 2) : (NB <= 4 ? 4 : 3); }
+// shared memory: vectors (q or nc long) | partial sums | couplings
+template <typename T, int MODE, int NB>
+constexpr size_t cr_smem(int q, int nc) {
+    return sizeof(cpx_t<T>) * ((size_t)cr_vecs<MODE>() * NB * (MODE == 6 ? nc : q) + (size_t)kMvThreads * NB +
+                               (size_t)cr_tabs<MODE>() * 6 * q);
 }
 
-// level 0 backward, odd blocks: x_j = y_j - D^{-1} (W_j x_{j-1} + E_j x_{j+1})
-template <typename T, int RPT, int NB>
-__global__ void __launch_bounds__(kMvThreads, NB >= 4 ? 2 : 1) k_cr_l0_back(int q, int nblk, const cpx_t<T>* __restrict__ cw,
-                                                          const cpx_t<T>* __restrict__ ce, Pool<T> pool,
-                                                          size_t off_dinv, cpx_t<T>* __restrict__ x, size_t SB,
-                                                          int nb) {
+template <typename T, int MODE, int NB>
+__global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(CrStep<T> a) {
     using C = cpx_t<T>;
+    constexpr int NM = cr_mats<MODE>(), NV = cr_vecs<MODE>(), PF = cr_prefetch<T, MODE>();
+    constexpr bool kEarly = sizeof(T) == 4 && NB == 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* vt = reinterpret_cast<C*>(smem_raw);   // [NB][q]
-    C* red = vt + (size_t)NB * q;             // [kMvWarps][NB][q]
-    const int o = blockIdx.x;
-    const int j = 2 * o + 1;
-    const C* wj = cw + (size_t)j * 3 * q;
-    const C* ej = ce + (size_t)j * 3 * q;
-    for (int e = threadIdx.x; e < NB * q; e += kMvThreads) {
-        const int b = e / q, r = e % q;
-        C acc = czero<C>();
-        if (b < nb) {
-            const C* xb = x + (size_t)b * SB;
+    if (kEarly) pdl_trigger();
+    const int q = a.q, n = a.src.n, ncol = MODE == 6 ? a.nc : q;
+    C* vin = reinterpret_cast<C*>(smem_raw);     // [NV][NB][ncol]
+    C* red = vin + (size_t)NV * NB * ncol;       // [CG][NB][R]
+    C* tab = red + kMvThreads * NB;              // MODE 4, 5: [v][W, E][dz+1][q]
+    const int tid = threadIdx.x;
+    const int b0 = blockIdx.z * NB, nb = a.nb - b0 < NB ? a.nb - b0 : NB;
+    const C* pool = a.pool + blockIdx.y * a.pool_strip;
+    C* x = a.x + blockIdx.y * a.x_strip + (size_t)b0 * a.SB;
+    C* y = a.y + blockIdx.y * a.x_strip + (size_t)b0 * a.YB;
+    // block and matrices
+    const size_t qq = (size_t)q * q;
+    const size_t s = (size_t)q << a.k;           // elements between neighbouring blocks of the level
+    bool odd = MODE == 0 || MODE == 2 || MODE == 4;
+    int bid = blockIdx.x;
+    if ((MODE == 1 || MODE == 5) && bid >= a.nlead) {
+        odd = true;
+        bid -= a.nlead;
+    }
+    const int idx = MODE == 6 ? 0 : bid / a.S, sp = bid - idx * a.S;
+    const int j = 2 * idx + (odd ? 1 : 0);
+    const bool hw = j >= 1, he = j + 1 < a.nk;
+    const C* Ms[NM];
+    int vb[NV], nm = 1, nv = 1;                  // the vectors' blocks (level index), matrices, vectors
+    if (MODE == 6) {
+        Ms[0] = a.inv;
+        vb[0] = 0;
+    } else if (NM == 1 || (MODE != 2 && odd)) {
+        Ms[0] = pool + (a.off_a + idx) * qq;
+        vb[0] = j;
+    } else {                                     // the neighbours that exist
+        const C* M0 = pool + (a.off_b + idx) * qq;
+        const C* M1 = pool + (a.off_c + idx) * qq;
+        Ms[0] = hw ? M0 : M1;
+        vb[0] = hw ? j - 1 : j + 1;
+        nm = nv = (hw && he) ? 2 : 1;
+        Ms[NM - 1] = nm == 2 ? M1 : Ms[0];
+        vb[NM - 1] = nm == 2 ? j + 1 : vb[0];
+        if (MODE == 5) {
+            vb[NV - 1] = j;                      // the even update of the block itself, in slot 2
+            nv = 3;
+        }
+    }
+    const int R = a.R, r0 = sp * R, nr = (MODE == 6 ? a.nc : q) - r0 < R ? (MODE == 6 ? a.nc : q) - r0 : R;
+    const int CG = kMvThreads / R, cg = tid / R, rr = tid - cg * R;
+    const bool act = cg < CG && rr < nr;
+    C pre[PF][NM];
+    auto load_col = [&](C (&m)[NM], int c) {
 #pragma unroll
-            for (int dz = -1; dz <= 1; ++dz) {
-                const int rr = r + dz;
-                if (rr < 0 || rr >= q) continue;
-                acc = cfma(wj[(dz + 1) * q + r], xb[(size_t)(j - 1) * q + rr], acc);
-                if (j + 1 < nblk) acc = cfma(ej[(dz + 1) * q + r], xb[(size_t)(j + 1) * q + rr], acc);
+        for (int t = 0; t < NM; ++t)
+            m[t] = (act && c < ncol && t < nm) ? __ldg(&Ms[t][(size_t)c * ncol + r0 + rr]) : czero<C>();
+    };
+#pragma unroll
+    for (int u = 0; u < PF; ++u) load_col(pre[u], cg + u * CG);
+    if constexpr (cr_tabs<MODE>() > 0) {
+        for (int e = tid; e < cr_tabs<MODE>() * 6 * q; e += kMvThreads) {
+            const int v = e / (6 * q), w = e - v * 6 * q;
+            const bool use = MODE == 4 || (v < NM ? v < nm : nv == 3);
+            const size_t i = MODE == 4 ? (size_t)j : 2 * (size_t)(v == 0 ? vb[0] : (v == 1 ? vb[NM - 1] : j));
+            if (use) tab[e] = __ldg(w < 3 * q ? &a.cp.cw[i * 3 * q + w] : &a.cp.ce[i * 3 * q + (w - 3 * q)]);
+        }
+        __syncthreads();
+    }
+    pdl_wait();
+
+    // vectors, row r = tid % 128, members and slots alternating between the halves of the CTA
+    if constexpr (MODE == 6) {
+        for (int c = tid; c < ncol; c += kMvThreads) {
+            const int jb = c / q;
+            const size_t e = (((size_t)jb << a.c) - jb) * q + c;   // (jb << c) * q + c % q
+#pragma unroll
+            for (int b = 0; b < NB; ++b) vin[(size_t)b * ncol + c] = b < nb ? y[b * a.YB + e] : czero<C>();
+        }
+    } else {
+        const int r = tid & 127;
+#pragma unroll
+        for (int p = 0; p < NV * NB; ++p) {
+            const int v = p / NB, b = p % NB;
+            if ((p & 1) != (tid >> 7) || r >= q) continue;
+            C val = czero<C>();
+            if (b < nb && (v < nm || (MODE == 5 && v == 2 && nv == 3))) {
+                const C* xb = x + (size_t)b * a.SB;
+                if (MODE == 0) val = a.src.load(j, r, b0 + b);
+                if (MODE == 1 || MODE == 2 || MODE == 3) {
+                    val = xb[(size_t)vb[v < NM ? v : 0] * s + r];
+                    if (MODE == 2 || !(odd || MODE == 3)) val = -val;
+                }
+                if (MODE == 4) {   // -(W x_{j-1} + E x_{j+1})
+#pragma unroll
+                    for (int dz = -1; dz <= 1; ++dz) {
+                        const int rz = r + dz;
+                        if (rz < 0 || rz >= q) continue;
+                        val = cfma(tab[(dz + 1) * q + r], xb[(size_t)(j - 1) * q + rz], val);
+                        if (he) val = cfma(tab[(dz + 4) * q + r], xb[(size_t)(j + 1) * q + rz], val);
+                    }
+                    val = -val;
+                }
+                if (MODE == 5) {   // b' of level-0 block i
+                    const int i = 2 * vb[v];
+                    const C* tv = tab + (size_t)v * 6 * q;
+                    val = a.src.load(i, r, b0 + b);
+#pragma unroll
+                    for (int dz = -1; dz <= 1; ++dz) {
+                        const int rz = r + dz;
+                        if (rz < 0 || rz >= q) continue;
+                        if (i >= 1) val = cfms(tv[(dz + 1) * q + r], xb[(size_t)(i - 1) * q + rz], val);
+                        if (i + 1 < n) val = cfms(tv[(dz + 4) * q + r], xb[(size_t)(i + 1) * q + rz], val);
+                    }
+                    if (!odd && v < 2) val = -val;
+                }
             }
+            vin[(size_t)p * q + r] = val;
         }
-        vt[e] = -acc;
+        if ((MODE == 0 || MODE == 5) && sp == 0 && tid < nb) a.src.keep_trace(MODE == 0 ? j : 2 * j, b0 + tid);
+    }
+    // what the result is added to (the first of this thread's outputs: fetched ahead)
+    const int nout = nb * nr;
+    auto base_of = [&](int b, int r) {
+        if (MODE == 2) return y[(size_t)b * a.YB + (size_t)j * s + r];
+        if ((MODE == 1 && !odd) || MODE == 4) return x[(size_t)b * a.SB + (size_t)j * s + r];
+        return czero<C>();
+    };
+    C base = czero<C>();
+    if (tid < nout) base = base_of(NB == 1 ? 0 : tid / nr, r0 + (NB == 1 ? tid : tid % nr));
+    __syncthreads();
+    if (!kEarly && !(sizeof(T) == 8 && gridDim.x <= 304)) pdl_trigger();   // else at its end
+    C part[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) part[b] = czero<C>();
+    for (int c0 = cg; c0 < ncol; c0 += CG * PF) {
+#pragma unroll
+        for (int u = 0; u < PF; ++u) {
+            const int c = c0 + u * CG;
+            if (c < ncol) {
+#pragma unroll
+                for (int t = 0; t < NM; ++t)
+                    if (t < nm) {
+#pragma unroll
+                        for (int b = 0; b < NB; ++b)
+                            part[b] = cfma(pre[u][t], vin[((size_t)t * NB + b) * ncol + c], part[b]);
+                    }
+            }
+            load_col(pre[u], c + CG * PF);
+        }
+    }
+    if (act) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) red[((size_t)cg * NB + b) * R + rr] = part[b];
     }
     __syncthreads();
-    const C* M = pool.mat(off_dinv + o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    C part[RPT][NB];
-#pragma unroll
-    for (int kk = 0; kk < RPT; ++kk)
-#pragma unroll
-        for (int b = 0; b < NB; ++b) part[kk][b] = czero<C>();
+    // the CG partial sums in two stages (about sqrt(CG) dependent adds each, in a fixed order):
+    // FP64 adds take tens of cycles, and a chain of 32 of them 2 us
+    auto add_up = [&](int first, int step, int b, int rc) {
+        C sum = red[((size_t)first * NB + b) * R + rc];
 #pragma unroll 4
-    for (int c = warp; c < q; c += kMvWarps) {
-        C a[RPT];
-#pragma unroll
-        for (int kk = 0; kk < RPT; ++kk) {
-            const int r = lane + 32 * kk;
-            a[kk] = r < q ? __ldg(&M[(size_t)c * q + r]) : czero<C>();
+        for (int g = first + step; g < CG; g += step) sum = sum + red[((size_t)g * NB + b) * R + rc];
+        return sum;
+    };
+    const int G1 = CG >= 25 ? 6 : (CG >= 9 ? 4 : CG);
+    if (G1 < CG) {
+        for (int o = tid; o < G1 * nout; o += kMvThreads) {
+            const int g = o / nout, w = o - g * nout, b = NB == 1 ? 0 : w / nr, rc = w - b * nr;
+            red[((size_t)g * NB + b) * R + rc] = add_up(g, G1, b, rc);
         }
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const C vc = vt[(size_t)b * q + c];
-#pragma unroll
-            for (int kk = 0; kk < RPT; ++kk) part[kk][b] = cfma(a[kk], vc, part[kk][b]);
+        __syncthreads();
+    }
+    for (int o = tid; o < nout; o += kMvThreads) {
+        const int b = NB == 1 ? 0 : o / nr, rc = o - b * nr, r = r0 + rc;
+        C sum = red[(size_t)b * R + rc];
+#pragma unroll 6
+        for (int g = 1; g < G1; ++g) sum = sum + red[((size_t)g * NB + b) * R + rc];
+        C* xb = x + (size_t)b * a.SB;
+        C* yb = y + (size_t)b * a.YB;
+        if (o != tid) base = base_of(b, r);
+        if (MODE == 6) {
+            const int jb = r / q;
+            xb[(((size_t)jb << a.c) - jb) * q + r] = sum;
+        } else if (MODE == 1 || MODE == 5) {
+            const size_t e = (size_t)j * s + r;
+            if (odd) {
+                yb[e] = sum;
+            } else {
+                sum = (MODE == 5 ? vin[((size_t)2 * NB + b) * q + r] : base) + sum;
+                if (a.to_y) yb[e] = sum;
+                else xb[e] = sum;
+            }
+        } else if (MODE == 2 || MODE == 4) {
+            xb[(size_t)j * s + r] = base + sum;
+        } else {   // MODE 0, 3
+            xb[(size_t)j * s + r] = sum;
         }
     }
+}
+
+// Level-0 even blocks on their own (FP64): x_i = b_i - W_i y_{i-1} - E_i y_{i+1}, one thread per
+// row and member.  MODE 5 forms this up to three times per block and once per row chunk, which
+// FP32 does not notice; on the FP64 pipe it cost 7 us of a 150 us solve (400^2, q = 70), this
+// kernel about 2.
+template <typename T>
+__global__ void __launch_bounds__(128) k_cr_even(CrStep<T> a) {
+    const int i = 2 * blockIdx.x, b = blockIdx.y, q = a.q, n = a.src.n;
+    const int r = threadIdx.x < q ? threadIdx.x : q - 1;
+    const cpx_t<T>* wi = a.cp.cw + (size_t)i * 3 * q + r;
+    const cpx_t<T>* ei = a.cp.ce + (size_t)i * 3 * q + r;
+    cpx_t<T> w[3], e[3], xw[3], xe[3];
 #pragma unroll
-    for (int kk = 0; kk < RPT; ++kk) {
-        const int r = lane + 32 * kk;
-        if (r < q)
+    for (int d = 0; d < 3; ++d) {
+        w[d] = __ldg(&wi[(size_t)d * q]);
+        e[d] = __ldg(&ei[(size_t)d * q]);
+    }
+    pdl_trigger();
+    pdl_wait();
+    if (threadIdx.x >= q) return;
+    if (r == 0) a.src.keep_trace(i, b);
+    cpx_t<T>* xb = a.x + (size_t)b * a.SB;
 #pragma unroll
-            for (int b = 0; b < NB; ++b) red[((size_t)warp * NB + b) * q + r] = part[kk][b];
+    for (int d = 0; d < 3; ++d) {
+        const int rz = r + d - 1;
+        const bool in = rz >= 0 && rz < q;
+        xw[d] = in && i >= 1 ? xb[(size_t)(i - 1) * q + rz] : czero<cpx_t<T>>();
+        xe[d] = in && i + 1 < n ? xb[(size_t)(i + 1) * q + rz] : czero<cpx_t<T>>();
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nb * q; e += kMvThreads) {
-        const int b = e / q, r = e % q;
-        C sum = czero<C>();
-        for (int w = 0; w < kMvWarps; ++w) sum = sum + red[((size_t)w * NB + b) * q + r];
-        C* xj = x + (size_t)b * SB + (size_t)j * q;
-        xj[r] = xj[r] + sum;
+    cpx_t<T> val = a.src.load(i, r, b);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (r + d - 1 < 0 || r + d - 1 >= q) continue;
+        if (i >= 1) val = cfms(w[d], xw[d], val);
+        if (i + 1 < n) val = cfms(e[d], xe[d], val);
     }
+    xb[(size_t)i * q + r] = val;
+}
+
+// the identity, nc x nc per strip (the right-hand sides of the reduced inverse)
+__global__ void k_identity(size_t total, int nc, double2* A) {
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const size_t w = e % ((size_t)nc * nc);
+        A[e] = make_double2(w / nc == w % nc ? 1.0 : 0.0, 0.0);
+    }
+}
+__global__ void k_inverse32(size_t total, const double2* __restrict__ a, float2* __restrict__ b) {
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x)
+        b[e] = ccast<float2>(a[e]);
 }
 
 // level 0, even blocks: b_j -= W_j y_{j-1} + E_j y_{j+1} (tabulated tridiagonal couplings)
@@ -346,6 +510,40 @@ __global__ void __launch_bounds__(256) k_gather(StripGeom g, const cpx_t<T>* __r
     }
 }
 
+// The same tiles for all layers of a sweep at once, without the injections (the reduction
+// steps on the CUDA cores add them where level 0 reads the right-hand side): blockIdx.z =
+// member * L + layer.
+template <typename T, bool TR, typename GF = double2>
+__global__ void __launch_bounds__(256) k_gather_all(StripGeom g, int L, const GF* __restrict__ gf,
+                                                    cpx_t<T>* __restrict__ rhs, size_t SB) {
+    using C = cpx_t<T>;
+    __shared__ C tile[kGatherTile][kGatherTile + 1];   // [r - r0][i - i0]
+    const int q = g.q, n = g.n, E = g.E, t = g.t;
+    const int b = blockIdx.z / L, l = blockIdx.z - b * L;
+    const int i0 = blockIdx.x * kGatherTile, r0 = blockIdx.y * kGatherTile;
+    gf += (size_t)b * n * n;
+    rhs += (size_t)b * SB + (size_t)l * n * q;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const GF z0 = {};
+    GF v[kGatherTile / 8];
+#pragma unroll
+    for (int u = 0; u < kGatherTile / 8; ++u) {   // rows of Omega^l (E <= r < E + t), along r (TR) or x
+        const int i = i0 + (TR ? ty + 8 * u : tx), r = r0 + (TR ? tx : ty + 8 * u);
+        const size_t e = TR ? (size_t)i * n + (l * t - E + r) : (size_t)(l * t - E + r) * n + i;
+        v[u] = (r >= E && r < E + t && i < n) ? __ldg(&gf[e]) : z0;
+    }
+    if constexpr (!TR) {
+#pragma unroll
+        for (int u = 0; u < kGatherTile / 8; ++u) tile[ty + 8 * u][tx] = ccast<C>(v[u]);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < kGatherTile / 8; ++u) {   // strip columns, along r
+        const int i = i0 + ty + 8 * u, r = r0 + tx;
+        if (i < n && r < q) rhs[(size_t)i * q + r] = TR ? ccast<C>(v[u]) : tile[tx][ty + 8 * u];
+    }
+}
+
 // Upward sweep: sol = g^l (a device copy of rhs made just before) plus the injection
 // from the layer below, which touches only the two rows E - 1 and E; one thread per
 // (column i, row) of those, batch member b = blockIdx.y.
@@ -429,73 +627,90 @@ __global__ void k_strip_out(int n, int q, const cpx_t<T>* __restrict__ x, double
 
 StripGeom geom_of(const ls_handle* h) { return StripGeom{h->n, h->t, h->E, h->q, h->opts.shift / h->omega}; }
 
-// CTAs per block of a reduction step: levels with fewer blocks than about two per SM
-// split each block's columns over up to kCrSplitMax CTAs (at most kCrSplitCtas CTAs in all).
-// The handle's cr_split switches it off (1 CTA per block everywhere).
-constexpr int kCrSplitCtas = 304, kCrSplitMax = 8;
-int cr_split_of(const ls_handle* h, int nblk) {
-    if (!h->cr_split) return 1;
-    int S = kCrSplitCtas / (nblk > 0 ? nblk : 1);
-    return S < 1 ? 1 : (S > kCrSplitMax ? kCrSplitMax : S);
+// Row chunks per block of a reduction step: levels with few blocks are split until about
+// kCtas CTAs run, down to chunks of 8 rows (64 contiguous bytes of an FP32 column; 4 rows of
+// the reduced inverse in FP64).  FP64 steps are bound by the FP64 pipe of each SM, so they
+// are cut finer, for balance: one CTA per block left SMs with twice the others' work.  The
+// handle's cr_split switches the splitting off (1 CTA per block).
+template <typename T>
+void cr_split(const ls_handle* h, CrStep<T>& a, int rows, int blocks, int min_rows = 8) {
+    constexpr int kCtas = 608;
+    int S = h->cr_split ? kCtas / blocks : 1;
+    if (S > rows / min_rows) S = rows / min_rows;
+    if (S < (rows + kMvThreads - 1) / kMvThreads) S = (rows + kMvThreads - 1) / kMvThreads;   // R <= kMvThreads
+    a.R = (rows + S - 1) / S;
+    a.S = (rows + a.R - 1) / a.R;
 }
 
-template <typename T, int RPT, int NB>
-int cr_solve_rpt(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb) {
+// Unknowns of the reduced system whose inverse replaces the levels from c on.  Larger means
+// fewer dependent steps and more bytes a solve (nc^2 entries instead of about 2.5 q^2 per
+// block): 8 blocks of 84 rows are one 3.6 MB (FP32) product of 2.5 us instead of seven steps
+// of 2.8 us; 16 blocks would read 14 MB to save two more.
+constexpr int kInverseMax = 700;
+
+template <typename T, int MODE, int NB>
+int cr_launch(ls_handle* h, const CrStep<T>& a, unsigned grid, unsigned strips = 1, unsigned groups = 1) {
+    return ls_launch_pdl(h, k_cr_step<T, MODE, NB>, dim3(grid, strips, groups), dim3(kMvThreads),
+                         cr_smem<T, MODE, NB>(a.q, a.nc), a);
+}
+
+template <typename T, int NB>
+int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, const RhsSrc<T>& src) {
     using C = cpx_t<T>;
     const DirFactors& F = h->fac[dir];
     const int q = h->q, n = h->n;
     const size_t qq = (size_t)q * q;
-    const C* base;
-    if constexpr (sizeof(T) == 4) base = F.pool32;
-    else base = F.pool64;
-    Pool<T> pool{base + (size_t)l * F.mats_per_strip * qq, qq};
-    const int thr = (q + 31) / 32 * 32;
-    const size_t sm_step = (size_t)(3 + kMvWarps) * NB * sizeof(C) * q;
-    const size_t sm_back = (size_t)(1 + kMvWarps) * NB * sizeof(C) * q;
     const CrLevel& l0 = F.lev[0];
-    const C* cw = static_cast<const C*>(F.cw) + (size_t)l * n * 3 * q;
-    const C* ce = static_cast<const C*>(F.ce) + (size_t)l * n * 3 * q;
     const ls_handle::SweepLane& W = h->lanes[h->lane];
-    C* part = static_cast<C*>(W.cr_part);
-    unsigned* cnt = W.cr_cnt;
-    if (l0.nodd) {
-        const int S = cr_split_of(h, l0.nodd);
-        LS_LAUNCH(h, (k_cr_step<T, RPT, 0, NB>), l0.nodd * S, kMvThreads, sm_step, q, 0, l0.nk, pool, l0.off_dinv,
-                  (size_t)0, (size_t)0, x, SB, nb, S, part, cnt);
-    }
-    LS_LAUNCH(h, k_l0_even<T>, dim3(l0.neven, nb), thr, 0, q, n, cw, ce, x, SB);
-    for (int k = 1; k < F.K; ++k) {
+    CrStep<T> a{};
+    a.q = q;
+    if constexpr (sizeof(T) == 4) a.pool = F.pool32 + (size_t)l * F.mats_per_strip * qq;
+    else a.pool = F.pool64 + (size_t)l * F.mats_per_strip * qq;
+    a.x = x;
+    a.y = static_cast<C*>(W.cr_y);
+    a.SB = SB;
+    a.YB = (size_t)n * q;
+    a.nb = nb;
+    a.src = src;
+    a.cp = Couple<T>{static_cast<const C*>(F.cw) + (size_t)l * n * 3 * q,
+                     static_cast<const C*>(F.ce) + (size_t)l * n * 3 * q};
+    a.nc = F.inv_nc;
+    a.c = F.inv_c;
+    a.inv = static_cast<const C*>(F.inv) + (size_t)l * a.nc * a.nc;
+    auto level = [&](int k, int blocks) {
         const CrLevel& lv = F.lev[k];
-        const int S = cr_split_of(h, lv.neven);
-        LS_LAUNCH(h, (k_cr_step<T, RPT, 1, NB>), lv.neven * S, kMvThreads, sm_step, q, k, lv.nk, pool, (size_t)0,
-                  lv.off_f, lv.off_g, x, SB, nb, S, part, cnt);
+        a.k = k;
+        a.nk = lv.nk;
+        a.off_a = lv.off_dinv;
+        a.to_y = k == a.c - 1;
+        cr_split(h, a, q, blocks);
+        a.nlead = lv.neven * a.S;
+        return (unsigned)(blocks * a.S);
+    };
+    LS_TRY((cr_launch<T, 0, NB>(h, a, level(0, l0.nodd))));
+    for (int k = 1; k < a.c; ++k) {
+        const unsigned grid = level(k, F.lev[k].nk);
+        a.off_b = F.lev[k].off_f;
+        a.off_c = F.lev[k].off_g;
+        if (sizeof(T) == 4 && k == 1) {
+            LS_TRY((cr_launch<T, 5, NB>(h, a, grid)));
+            continue;
+        }
+        if (k == 1)
+            LS_TRY(ls_launch_pdl(h, k_cr_even<T>, dim3((unsigned)l0.neven, (unsigned)nb), dim3(128), 0, a));
+         LS_TRY((cr_launch<T, 1, NB>(h, a, grid)));
     }
-    {
-        const int S = cr_split_of(h, 1);
-        LS_LAUNCH(h, (k_cr_step<T, RPT, 3, NB>), S, kMvThreads, sm_step, q, 0, 1, pool, F.off_top, (size_t)0,
-                  (size_t)0, x, SB, nb, S, part, cnt);
+    cr_split(h, a, a.nc, 1, sizeof(T) == 8 ? 4 : 8);
+    LS_TRY((cr_launch<T, 6, NB>(h, a, (unsigned)a.S)));
+    for (int k = a.c - 1; k >= 1; --k) {
+        if (!F.lev[k].nodd) continue;
+        const unsigned grid = level(k, F.lev[k].nodd);
+        a.off_b = F.lev[k].off_p;
+        a.off_c = F.lev[k].off_q;
+        LS_TRY((cr_launch<T, 2, NB>(h, a, grid)));
     }
-    for (int k = F.K - 1; k >= 1; --k) {
-        const CrLevel& lv = F.lev[k];
-        if (!lv.nodd) continue;
-        const int S = cr_split_of(h, lv.nodd);
-        LS_LAUNCH(h, (k_cr_step<T, RPT, 2, NB>), lv.nodd * S, kMvThreads, sm_step, q, k, lv.nk, pool, lv.off_dinv,
-                  lv.off_p, lv.off_q, x, SB, nb, S, part, cnt);
-    }
-    if (l0.nodd)
-        LS_LAUNCH(h, (k_cr_l0_back<T, RPT, NB>), l0.nodd, kMvThreads, sm_back, q, n, cw, ce, pool, l0.off_dinv, x,
-                  SB, nb);
-    return LS_OK;
-}
-
-template <typename T, int NB>
-int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb) {
-    switch ((h->q + 31) / 32) {
-        case 1: return cr_solve_rpt<T, 1, NB>(h, dir, l, x, SB, nb);
-        case 2: return cr_solve_rpt<T, 2, NB>(h, dir, l, x, SB, nb);
-        case 3: return cr_solve_rpt<T, 3, NB>(h, dir, l, x, SB, nb);
-        default: return cr_solve_rpt<T, 4, NB>(h, dir, l, x, SB, nb);
-    }
+    const unsigned grid = level(0, l0.nodd);
+    return cr_launch<T, 4, NB>(h, a, grid);
 }
 
 // The same local solve with the reduction steps on the tensor cores (ls_cr_mma.cu):
@@ -529,19 +744,61 @@ int cr_solve_tc(ls_handle* h, int dir, int l, float2* x, size_t SB, int nb) {
     return LS_OK;
 }
 
-// The batch template is the smallest supported NB >= nb (FP64 keeps NB <= 4 for registers).
+// Where the reduction steps of a pass over nb right-hand sides run: on the tensor cores
+// always (cr_tc 2), or for batches past the CUDA-core steps' sweet spot (cr_tc 1: at least 5
+// right-hand sides; a one-matrix product per step does not fill them)
 template <typename T>
-int cr_solve(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb) {
-    if constexpr (sizeof(T) == 4) {
-        // tensor cores: always (cr_tc 2), or for batches past the CUDA-core steps' sweet spot
-        // (cr_tc 1: at least 5 right-hand sides; a one-matrix product per step does not fill them)
-        if (h->tc_ready && (h->cr_tc == 2 || (h->cr_tc == 1 && nb >= 5))) return cr_solve_tc(h, dir, l, x, SB, nb);
-    }
-    if (nb <= 1) return cr_solve_nb<T, 1>(h, dir, l, x, SB, nb);
-    if (nb <= 2) return cr_solve_nb<T, 2>(h, dir, l, x, SB, nb);
-    if (nb <= 4) return cr_solve_nb<T, 4>(h, dir, l, x, SB, nb);
-    if constexpr (sizeof(T) == 4) return cr_solve_nb<T, 8>(h, dir, l, x, SB, nb);
+bool cr_on_tensor_cores(const ls_handle* h, int nb) {
+    return sizeof(T) == 4 && h->tc_ready && (h->cr_tc == 2 || (h->cr_tc == 1 && nb >= 5));
+}
+
+// Local solve on the CUDA cores: x = (C^l)^{-1} of the right-hand side src (which x must not
+// overlap).  The batch template is the smallest supported NB >= nb (FP64 keeps NB <= 4 for
+// registers).
+template <typename T>
+int cr_solve(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, const RhsSrc<T>& src) {
+    if (nb <= 1) return cr_solve_nb<T, 1>(h, dir, l, x, SB, nb, src);
+    if (nb <= 2) return cr_solve_nb<T, 2>(h, dir, l, x, SB, nb, src);
+    if (nb <= 4) return cr_solve_nb<T, 4>(h, dir, l, x, SB, nb, src);
+    if constexpr (sizeof(T) == 4) return cr_solve_nb<T, 8>(h, dir, l, x, SB, nb, src);
     return LS_EINVAL;
+}
+
+// The downward and upward sweeps with the local solves on the tensor cores (solutions in the
+// lane's ssol; see sweep_impl).
+template <typename GF>
+int sweep_tc(ls_handle* h, int dir, const GF* g, int nb, bool tr) {
+    const int n = h->n, q = h->q, L = h->L;
+    const size_t sstride = (size_t)n * q;
+    const size_t SB = (size_t)L * sstride, TB = (size_t)L * n;
+    const ls_handle::SweepLane& W = h->lanes[h->lane];
+    float2* rhs = static_cast<float2*>(W.srhs);
+    float2* sol = static_cast<float2*>(W.ssol);
+    float2* trc = static_cast<float2*>(W.strace);
+    const float2* cinj = static_cast<const float2*>(h->fac[dir].cinj);
+    const StripGeom geo = geom_of(h);
+    const dim3 gg((unsigned)((n + kGatherTile - 1) / kGatherTile), (unsigned)((q + kGatherTile - 1) / kGatherTile), nb);
+    const dim3 gb(kGatherTile, 8);
+    for (int l = L - 1; l >= 0; --l) {  // downward sweep
+        const float2* above = l < L - 1 ? sol + (l + 1) * sstride : nullptr;
+        float2* tabove = l < L - 1 ? trc + (size_t)(l + 1) * n : nullptr;
+        if (tr)
+            LS_LAUNCH(h, (k_gather<float, true, GF>), gg, gb, 0, geo, cinj, l, g, rhs + l * sstride, sol + l * sstride,
+                      above, tabove, SB, TB);
+        else
+            LS_LAUNCH(h, (k_gather<float, false, GF>), gg, gb, 0, geo, cinj, l, g, rhs + l * sstride, sol + l * sstride,
+                      above, tabove, SB, TB);
+        LS_TRY(cr_solve_tc(h, dir, l, sol + l * sstride, SB, nb));
+    }
+    const dim3 gi((unsigned)((2 * n + 255) / 256), nb);
+    for (int l = 1; l < L; ++l) {  // upward sweep: sol = rhs, then the two injected rows
+        LS_CUDA(cudaMemcpy2DAsync(sol + l * sstride, sizeof(float2) * SB, rhs + l * sstride, sizeof(float2) * SB,
+                                  sizeof(float2) * sstride, nb, cudaMemcpyDeviceToDevice, h->stream));
+        LS_LAUNCH(h, k_inject_up<float>, gi, 256, 0, geo, cinj, l, rhs + l * sstride, sol + l * sstride,
+                  sol + (l - 1) * sstride, trc + (size_t)l * n, SB, TB);
+        LS_TRY(cr_solve_tc(h, dir, l, sol + l * sstride, SB, nb));
+    }
+    return LS_OK;
 }
 
 // tr: g and v are fields of the other direction's grid (read and written transposed);
@@ -562,24 +819,34 @@ int sweep_impl(ls_handle* h, int dir, const GF* g, OF* v, int nb, bool tr = fals
     const StripGeom geo = geom_of(h);
     const dim3 gg((unsigned)((n + kGatherTile - 1) / kGatherTile), (unsigned)((q + kGatherTile - 1) / kGatherTile), nb);
     const dim3 gb(kGatherTile, 8);
-    for (int l = L - 1; l >= 0; --l) {  // downward sweep
-        if (tr)
-            LS_LAUNCH(h, (k_gather<T, true, GF>), gg, gb, 0, geo, static_cast<const C*>(F.cinj), l, g, rhs + l * sstride,
-                      sol + l * sstride, l < L - 1 ? sol + (l + 1) * sstride : (const C*)nullptr,
-                      l < L - 1 ? trc + (size_t)(l + 1) * n : (C*)nullptr, SB, TB);
-        else
-            LS_LAUNCH(h, (k_gather<T, false, GF>), gg, gb, 0, geo, static_cast<const C*>(F.cinj), l, g, rhs + l * sstride,
-                      sol + l * sstride, l < L - 1 ? sol + (l + 1) * sstride : (const C*)nullptr,
-                      l < L - 1 ? trc + (size_t)(l + 1) * n : (C*)nullptr, SB, TB);
-        LS_TRY(cr_solve<T>(h, dir, l, sol + l * sstride, SB, nb));
+    const C* cinj = static_cast<const C*>(F.cinj);
+    bool tc = false;
+    if constexpr (sizeof(T) == 4) {
+        tc = cr_on_tensor_cores<T>(h, nb);
+        if (tc) LS_TRY((sweep_tc<GF>(h, dir, g, nb, tr)));
     }
-    const dim3 gi((unsigned)((2 * n + 255) / 256), nb);
-    for (int l = 1; l < L; ++l) {  // upward sweep: sol = rhs, then the two injected rows
-        LS_CUDA(cudaMemcpy2DAsync(sol + l * sstride, sizeof(C) * SB, rhs + l * sstride, sizeof(C) * SB,
-                                  sizeof(C) * sstride, nb, cudaMemcpyDeviceToDevice, h->stream));
-        LS_LAUNCH(h, k_inject_up<T>, gi, 256, 0, geo, static_cast<const C*>(F.cinj), l, rhs + l * sstride,
-                  sol + l * sstride, sol + (l - 1) * sstride, trc + (size_t)l * n, SB, TB);
-        LS_TRY(cr_solve<T>(h, dir, l, sol + l * sstride, SB, nb));
+    if (!tc) {
+        const dim3 ga(gg.x, gg.y, (unsigned)(nb * L));
+        if (tr) LS_LAUNCH(h, (k_gather_all<T, true, GF>), ga, gb, 0, geo, L, g, rhs, SB);
+        else LS_LAUNCH(h, (k_gather_all<T, false, GF>), ga, gb, 0, geo, L, g, rhs, SB);
+        RhsSrc<T> src{};
+        src.SB = SB;
+        src.TB = TB;
+        src.n = n;
+        src.q = q;
+        src.E = h->E;
+        src.t = h->t;
+        auto layer = [&](int l, bool up) {
+            src.rhs = rhs + l * sstride;
+            src.inj = cinj + (size_t)l * 12 * n;
+            src.above = l < L - 1 ? sol + (l + 1) * sstride : nullptr;
+            src.below = up ? sol + (l - 1) * sstride : nullptr;
+            src.tself = trc + (size_t)l * n;
+            src.tsave = !up && l < L - 1 ? trc + (size_t)(l + 1) * n : nullptr;
+            return cr_solve<T>(h, dir, l, sol + l * sstride, SB, nb, src);
+        };
+        for (int l = L - 1; l >= 0; --l) LS_TRY(layer(l, false));   // downward sweep
+        for (int l = 1; l < L; ++l) LS_TRY(layer(l, true));         // upward sweep
     }
     const size_t N = (size_t)n * n;
     if (tr && add) {
@@ -591,35 +858,31 @@ int sweep_impl(ls_handle* h, int dir, const GF* g, OF* v, int nb, bool tr = fals
     return LS_OK;
 }
 
-template <typename T>
-int smem_optin(int q) {
-    using C = cpx_t<T>;
-    const int rpt = (q + 31) / 32;
-    const size_t s8 = (size_t)(3 + kMvWarps) * 8 * sizeof(C) * q, s4 = (size_t)(3 + kMvWarps) * 4 * sizeof(C) * q;
-    const size_t big = sizeof(T) == 4 ? s8 : s4;
-    if (big <= 48 * 1024) return LS_OK;
-#define LS_OPTIN(R, NB)                                                                                           \
-    do {                                                                                                          \
-        const size_t sz = (size_t)(3 + kMvWarps) * NB * sizeof(C) * q;                                            \
-        LS_CUDA(cudaFuncSetAttribute(k_cr_step<T, R, 0, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz)); \
-        LS_CUDA(cudaFuncSetAttribute(k_cr_step<T, R, 1, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz)); \
-        LS_CUDA(cudaFuncSetAttribute(k_cr_step<T, R, 2, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz)); \
-        LS_CUDA(cudaFuncSetAttribute(k_cr_step<T, R, 3, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz)); \
-        LS_CUDA(cudaFuncSetAttribute(k_cr_l0_back<T, R, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz)); \
-    } while (0)
-#define LS_OPTIN_R(NB)                  \
-    switch (rpt) {                      \
-        case 1: LS_OPTIN(1, NB); break; \
-        case 2: LS_OPTIN(2, NB); break; \
-        case 3: LS_OPTIN(3, NB); break; \
-        default: LS_OPTIN(4, NB); break; \
-    }
-    LS_OPTIN_R(2);
-    LS_OPTIN_R(4);
-    if constexpr (sizeof(T) == 4) LS_OPTIN_R(8);
-#undef LS_OPTIN_R
-#undef LS_OPTIN
+template <typename T, int NB, int... MODES>
+int smem_optin_modes(int q) {
+    cudaError_t e = cudaSuccess;
+    auto one = [&](auto kern, size_t sz) {
+        if (e == cudaSuccess && sz > 48 * 1024)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz);
+    };
+    (one(k_cr_step<T, MODES, NB>, cr_smem<T, MODES, NB>(q, kInverseMax)), ...);
+    LS_CUDA(e);
     return LS_OK;
+}
+template <typename T, int NB>
+int smem_optin_nb(int q) { return smem_optin_modes<T, NB, 0, 1, 2, 4, 5, 6>(q); }
+int smem_optin(bool mixed, int q) {
+    if (mixed) {
+        LS_TRY((smem_optin_nb<float, 1>(q)));
+        LS_TRY((smem_optin_nb<float, 2>(q)));
+        LS_TRY((smem_optin_nb<float, 4>(q)));
+        LS_TRY((smem_optin_nb<float, 8>(q)));
+    } else {
+        LS_TRY((smem_optin_nb<double, 1>(q)));
+        LS_TRY((smem_optin_nb<double, 2>(q)));
+        LS_TRY((smem_optin_nb<double, 4>(q)));
+    }
+    return smem_optin_modes<double, 8, 1, 2, 3>(q);   // the reduced inverse
 }
 
 }  // namespace
@@ -643,9 +906,9 @@ int ls_sweep_reserve(ls_handle* h, int nb) {
     const size_t cnt = (size_t)h->L * h->n * h->q * nb;
     const size_t es = h->prec == LS_MIXED ? sizeof(float2) : sizeof(double2);
     const size_t N = (size_t)h->n * h->n;
-    void* ptrs[] = {W.srhs, W.ssol, W.strace, W.vtmp, W.bd_in, W.bd_out};
+    void* ptrs[] = {W.srhs, W.ssol, W.strace, W.vtmp, W.bd_in, W.bd_out, W.cr_y};
     for (void* p : ptrs) cudaFree(p);
-    W.srhs = W.ssol = W.strace = W.vtmp = nullptr;
+    W.srhs = W.ssol = W.strace = W.vtmp = W.cr_y = nullptr;
     W.bd_in = W.bd_out = nullptr;
     W.nb_cap = 0;
     LS_CUDA(cudaMalloc(&W.srhs, es * cnt));
@@ -654,11 +917,7 @@ int ls_sweep_reserve(ls_handle* h, int nb) {
     LS_CUDA(cudaMalloc(&W.vtmp, sizeof(double2) * N * 4 * nb));
     LS_CUDA(cudaMalloc(&W.bd_in, sizeof(double2) * N * nb));
     LS_CUDA(cudaMalloc(&W.bd_out, sizeof(double2) * N * nb));
-    if (!W.cr_part) {  // split-level partial sums (kCrSplitCtas CTAs x 8 vectors x q) and counters
-        LS_CUDA(cudaMalloc(&W.cr_part, sizeof(double2) * kCrSplitCtas * 8 * h->q));
-        LS_CUDA(cudaMalloc(&W.cr_cnt, sizeof(unsigned) * kCrSplitCtas));
-        LS_CUDA(cudaMemset(W.cr_cnt, 0, sizeof(unsigned) * kCrSplitCtas));
-    }
+    LS_CUDA(cudaMalloc(&W.cr_y, es * (size_t)h->n * h->q * nb));
     W.nb_cap = nb;
     return LS_OK;
 }
@@ -666,7 +925,7 @@ int ls_sweep_reserve(ls_handle* h, int nb) {
 void ls_lanes_free(ls_handle* h) {
     for (auto& W : h->lanes) {
         lane_graphs_free(W);
-        void* ptrs[] = {W.srhs, W.ssol, W.strace, W.vtmp, W.bd_in, W.bd_out, W.cr_part, W.cr_cnt, W.dense_part};
+        void* ptrs[] = {W.srhs, W.ssol, W.strace, W.vtmp, W.bd_in, W.bd_out, W.cr_y, W.dense_part};
         for (void* p : ptrs) cudaFree(p);
         if (W.stream) cudaStreamDestroy(W.stream);
         if (W.done) cudaEventDestroy(W.done);
@@ -676,9 +935,83 @@ void ls_lanes_free(ls_handle* h) {
     h->ev_fork = nullptr;
 }
 
+// The inverse of the reduced system of level c (the first level >= 2 with at most kInverseMax
+// unknowns; level K - 1 has two blocks, so there is one) of every strip of a direction: the
+// steps of the levels from c on, in FP64, applied to the identity's columns in place -- every
+// strip and column in the same launches.  Stored in the solves' precision.  Called by
+// ls_factor once the factors in pool64 are complete (and the stream idle: the steps read
+// factors ahead of their turn).
+int ls_cr_inverse_build(ls_handle* h, int dir) {
+    DirFactors& F = h->fac[dir];
+    const int q = h->q, L = h->L;
+    int c = 2;
+    while (c < F.K - 1 && F.lev[c].nk * q > kInverseMax) ++c;
+    const int nc = F.lev[c].nk * q;
+    const size_t per = (size_t)nc * nc, total = per * L;
+    double2 *A = nullptr, *y = nullptr;
+    LS_CUDA(cudaMalloc(&A, sizeof(double2) * total));
+    int rc = LS_OK;
+    do {
+        if (cudaMalloc(&y, sizeof(double2) * total) != cudaSuccess) { rc = LS_ENOMEM; break; }
+        k_identity<<<1216, 256, 0, h->stream>>>(total, nc, A);
+        h->launches++;
+        CrStep<double> a{};
+        a.q = q;
+        a.pool = F.pool64;
+        a.pool_strip = F.mats_per_strip * (size_t)q * q;
+        a.x = A;
+        a.y = y;
+        a.SB = a.YB = nc;
+        a.x_strip = per;
+        a.nb = nc;
+        a.S = 1;
+        a.R = q;
+        const unsigned groups = (unsigned)((nc + 7) / 8);
+        for (int k = c; k < F.K && rc == LS_OK; ++k) {
+            const CrLevel& lv = F.lev[k];
+            a.k = k - c;
+            a.nk = lv.nk;
+            a.off_a = lv.off_dinv;
+            a.off_b = lv.off_f;
+            a.off_c = lv.off_g;
+            a.nlead = lv.neven;
+            rc = cr_launch<double, 1, 8>(h, a, (unsigned)lv.nk, (unsigned)L, groups);
+        }
+        if (rc != LS_OK) break;
+        a.k = 0;
+        a.nk = 1;
+        a.off_a = F.off_top;
+        if ((rc = cr_launch<double, 3, 8>(h, a, 1, (unsigned)L, groups)) != LS_OK) break;
+        for (int k = F.K - 1; k >= c && rc == LS_OK; --k) {
+            const CrLevel& lv = F.lev[k];
+            a.k = k - c;
+            a.nk = lv.nk;
+            a.off_b = lv.off_p;
+            a.off_c = lv.off_q;
+            if (lv.nodd) rc = cr_launch<double, 2, 8>(h, a, (unsigned)lv.nodd, (unsigned)L, groups);
+        }
+        if (rc != LS_OK) break;
+        if (h->prec == LS_MIXED) {
+            if (cudaMalloc(&F.inv, sizeof(float2) * total) != cudaSuccess) { rc = LS_ENOMEM; break; }
+            k_inverse32<<<1216, 256, 0, h->stream>>>(total, A, static_cast<float2*>(F.inv));
+            h->launches++;
+        } else {
+            F.inv = A;
+            A = nullptr;
+        }
+        F.inv_c = c;
+        F.inv_nc = nc;
+        cudaError_t e = cudaPeekAtLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) rc = ls_cuda_fail(e);
+    } while (0);
+    cudaFree(A);
+    cudaFree(y);
+    return rc;
+}
+
 int ls_sweep_alloc(ls_handle* h) {
-    if (h->prec == LS_MIXED) LS_TRY(smem_optin<float>(h->q));
-    else LS_TRY(smem_optin<double>(h->q));
+    LS_TRY(smem_optin(h->prec == LS_MIXED, h->q));
     for (int k = 1; k < ls_handle::kLanes; ++k) {
         LS_CUDA(cudaStreamCreateWithFlags(&h->lanes[k].stream, cudaStreamNonBlocking));
         LS_CUDA(cudaEventCreateWithFlags(&h->lanes[k].done, cudaEventDisableTiming));
@@ -885,21 +1218,33 @@ int ls_bd_cap(const ls_handle* h) {
     return h->tc_ready && h->cr_tc ? ls_cr_tc_max_nb(h) : 8;
 }
 
+template <typename T>
+static int strip_solve(ls_handle* h, int dir, int layer, const double2* b, double2* x, unsigned nblk, size_t SB) {
+    using C = cpx_t<T>;
+    const int n = h->n, q = h->q;
+    C* sol = static_cast<C*>(h->lanes[0].ssol);
+    C* rhs = static_cast<C*>(h->lanes[0].srhs);
+    if (cr_on_tensor_cores<T>(h, 1)) {   // in place
+        LS_LAUNCH(h, k_strip_in<T>, nblk, 256, 0, n, q, b, sol);
+        if constexpr (sizeof(T) == 4) LS_TRY(cr_solve_tc(h, dir, layer, sol, SB, 1));
+    } else {
+        LS_LAUNCH(h, k_strip_in<T>, nblk, 256, 0, n, q, b, rhs);
+        RhsSrc<T> src{};
+        src.rhs = rhs;
+        src.SB = SB;
+        src.n = n;
+        src.q = q;
+        LS_TRY(cr_solve<T>(h, dir, layer, sol, SB, 1, src));
+    }
+    LS_LAUNCH(h, k_strip_out<T>, nblk, 256, 0, n, q, sol, x);
+    return LS_OK;
+}
+
 int ls_strip_solve(ls_handle* h, int dir, int layer, const double2* b, double2* x) {
     const int n = h->n, q = h->q;
     const size_t cnt = (size_t)n * q;
     const unsigned nblk = (unsigned)((cnt + 255) / 256);
     const size_t SB = (size_t)h->L * cnt;
-    if (h->prec == LS_MIXED) {
-        float2* s = static_cast<float2*>(h->lanes[0].ssol);
-        LS_LAUNCH(h, k_strip_in<float>, nblk, 256, 0, n, q, b, s);
-        LS_TRY(cr_solve<float>(h, dir, layer, s, SB, 1));
-        LS_LAUNCH(h, k_strip_out<float>, nblk, 256, 0, n, q, s, x);
-    } else {
-        double2* s = static_cast<double2*>(h->lanes[0].ssol);
-        LS_LAUNCH(h, k_strip_in<double>, nblk, 256, 0, n, q, b, s);
-        LS_TRY(cr_solve<double>(h, dir, layer, s, SB, 1));
-        LS_LAUNCH(h, k_strip_out<double>, nblk, 256, 0, n, q, s, x);
-    }
-    return LS_OK;
+    return h->prec == LS_MIXED ? strip_solve<float>(h, dir, layer, b, x, nblk, SB)
+                               : strip_solve<double>(h, dir, layer, b, x, nblk, SB);
 }
