@@ -227,12 +227,13 @@ int ls_solve_group(int nprob, ls_handle* const* hs, const ls_c64* const* f, doub
  * this handle with incident-wave right-hand sides of its own problem:
  *   - the FFT tile shape of the FP32 / mixed LS-apply (column pass): fft_variant
  *     0 = radix-16 transforms on 1-column tiles, 3 CTAs per SM; 2 = radix-16 on
- *     2-column tiles (the default); 3 = radix-16 on 1-column tiles, 2 CTAs per SM;
+ *     2-column tiles; 3 = radix-16 on 1-column tiles, 2 CTAs per SM;
  *     4 = radix-8 per thread on 1-column tiles; 5 = radix-8 per thread on
  *     2-column tiles; 6, 7 = shapes 2 and 5 with the column tiles moved between
  *     HBM and shared memory by TMA; 8 = shape 6 with the two columns of a tile in
- *     packed FP32x2 instructions (0 and 2..8 need 256 <= P <= 4096); 1 = the
- *     generic radix-8 transforms on 4-column tiles;
+ *     packed FP32x2 instructions (4 needs 32 <= P <= 4096, 0 and the other shapes but
+ *     1 need 256 <= P <= 4096); 1 = the generic radix-8 transforms on 4-column tiles.  A
+ *     handle starts with 4 up to P = 512 and with 8 above;
  *   - the band-block batching of Algorithm 2 for nrhs right-hand sides: bd_chunk
  *     = right-hand sides per pass over the local-solve factors (1, 2, 4, 8;
  *     FP64 up to 4), chunks running concurrently on separate streams, and
@@ -260,7 +261,7 @@ typedef struct {
 int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out);
 
 /* ls_set_shapes -- pin the two shape choices (e.g. from an earlier ls_autotune):
- * fft_variant 0..8 as above (a radix-16/8 shape on a P outside 256..4096 falls back
+ * fft_variant 0..8 as above (a radix-16/8 shape on a P outside its range falls back
  * to the generic one), bd_chunk 1..32 with the tensor-core steps, 1..8 on the CUDA
  * cores (FP64: 1..4), or 0 for the largest.  LS_EINVAL otherwise.  Results agree up to
  * rounding whichever shapes are set. */

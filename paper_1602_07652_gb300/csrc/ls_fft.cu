@@ -499,6 +499,7 @@ int ls_fft_init(ls_handle* h) {
     LS_TRY(allow_smem(k_rows_fwd<float, E32, SrcMU<float, double2>>, row_smem32(P)));
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<float2>>, row_smem32(P)));
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<double2>>, row_smem32(P)));
+    h->fft_variant = ls_fft16_default(h);
     return ls_fft16_init(h);
 }
 
@@ -568,7 +569,7 @@ int ls_apply_df(ls_handle* h, const double2* u, double2* y) {
 }
 
 int ls_apply32(ls_handle* h, const float2* u, float2* y) {
-    if (h->fft_variant != 1 && ls_fft16_supported(h)) return ls_apply32_fft16(h, u, y, h->fft_variant);
+    if (ls_fft16_supported(h, h->fft_variant)) return ls_apply32_fft16(h, u, y, h->fft_variant);
     const int n = h->n, P = h->P;
     const FftPlan& pl = h->plan32;
     float2* X = static_cast<float2*>(h->fftws);
@@ -584,7 +585,7 @@ int ls_apply32(ls_handle* h, const float2* u, float2* y) {
 }
 
 int ls_apply_mx(ls_handle* h, const double2* u, double2* y) {
-    if (h->fft_variant != 1 && ls_fft16_supported(h)) return ls_apply_mx_fft16(h, u, y, h->fft_variant);
+    if (ls_fft16_supported(h, h->fft_variant)) return ls_apply_mx_fft16(h, u, y, h->fft_variant);
     const int n = h->n, P = h->P;
     const FftPlan& pl = h->plan32;
     float2* X = static_cast<float2*>(h->fftws);

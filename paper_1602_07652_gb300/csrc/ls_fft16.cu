@@ -26,6 +26,14 @@
 // on expiry the tile is written as NaN and a device counter is raised, so the
 // solver's residual checks see it).  Shape 8 also keeps the two columns of a
 // tile in packed FP32x2 registers, one instruction per operation on both.
+//
+// The three passes are launched programmatically, each letting its successor start when only
+// its stores are left: a kernel boundary on a stream costs about 2 us, which was a third of a
+// small call, and the column pass fetches its Ghat rows meanwhile.  Triggering at a pass's
+// start instead crowds the SMs that are idle then (512^2: 24 us against 15).  With this, the
+// kernels for 32 <= P < 256 and the default tile shapes (ls_fft16_default), back-to-back calls
+// went from 20.5 to 6.3 us (64^2), 21.6 to 8.9 (256^2), 24.6 to 14.9 (512^2), 57.7 to 41.6
+// (1024^2) and 199 to 141 us (2048^2).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -35,13 +43,16 @@
 
 namespace {
 
-// Geometry of a transform of P = 2^LP points, E = 2^LE elements per thread.
-template <int LP, int LE>
+// Geometry of a transform of P = 2^LP points, E = 2^LE elements per thread, CTAs of at least
+// MINT threads: 64 for the passes without TMA (a short transform's CTA then holds few of
+// them, so the call spreads over more SMs and a barrier joins two warps), 256 with it.
+constexpr int kSmallCta = 64, kTmaCta = 256;
+template <int LP, int LE, int MINT = kSmallCta>
 struct Geo {
     static constexpr int P = 1 << LP;
     static constexpr int E = 1 << LE;
-    static constexpr int T = P / E;                      // threads per transform
-    static constexpr int THREADS = T >= 256 ? T : 256;   // CTA size
+    static constexpr int T = P / E;                        // threads per transform
+    static constexpr int THREADS = T >= MINT ? T : MINT;   // CTA size
     static constexpr int G = THREADS / T;                // transforms per CTA
     static constexpr int NS = (LP + LE - 1) / LE;        // stages
     static constexpr int LRL = LP - LE * (NS - 1);       // log2 radix of the last forward stage
@@ -83,18 +94,23 @@ __device__ __forceinline__ void twiddle(V (&v)[CW][E], int e, int k, const float
     constexpr int SH = LP - LS - LR;
     float2 w[16];
     w[1] = ld_tw<DIR>(tw, k << SH);
-    if (R > 2) w[2] = ld_tw<DIR>(tw, (2 * k) << SH);
-    if (R > 4) w[4] = ld_tw<DIR>(tw, (4 * k) << SH);
-    if (R > 8) w[8] = ld_tw<DIR>(tw, (8 * k) << SH);
-    if (R > 2) w[3] = w[2] * w[1];
-    if (R > 4) {
-        w[5] = w[4] * w[1];
-        w[6] = w[4] * w[2];
-        w[7] = w[4] * w[3];
-    }
-    if (R > 8) {
+    if constexpr (LP < 8) {   // short transforms wait on latency, not on load slots: all from the table
 #pragma unroll
-        for (int r = 9; r < 16; ++r) w[r] = w[8] * w[r - 8];
+        for (int r = 2; r < R; ++r) w[r] = ld_tw<DIR>(tw, (r * k) << SH);
+    } else {
+        if (R > 2) w[2] = ld_tw<DIR>(tw, (2 * k) << SH);
+        if (R > 4) w[4] = ld_tw<DIR>(tw, (4 * k) << SH);
+        if (R > 8) w[8] = ld_tw<DIR>(tw, (8 * k) << SH);
+        if (R > 2) w[3] = w[2] * w[1];
+        if (R > 4) {
+            w[5] = w[4] * w[1];
+            w[6] = w[4] * w[2];
+            w[7] = w[4] * w[3];
+        }
+        if (R > 8) {
+#pragma unroll
+            for (int r = 9; r < 16; ++r) w[r] = w[8] * w[r - 8];
+        }
     }
 #pragma unroll
     for (int c = 0; c < CW; ++c)
@@ -303,6 +319,7 @@ __global__ void __launch_bounds__(Geo<LP, 4>::THREADS) k_rows16_fwd(int nrows, i
     float2* buf = reinterpret_cast<float2*>(smem_raw) + grp * Gm::SLOTS;
     const int z = blockIdx.x * Gm::G + grp;
     const bool live = z < nrows;
+    pdl_wait();
     float2 v[1][E];
 #pragma unroll
     for (int t = 0; t < E / 2; ++t) {
@@ -310,6 +327,7 @@ __global__ void __launch_bounds__(Geo<LP, 4>::THREADS) k_rows16_fwd(int nrows, i
         v[0][t] = (live && x < nin) ? src.template load<float2>(z, x) : make_float2(0.f, 0.f);
     }
     fwd_stages<LP, 4, 0, true>(v, buf, j, tw);
+    pdl_trigger();
     if (!live) return;
     float2* o = X + (size_t)z * P;
 #pragma unroll
@@ -347,6 +365,7 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16(int nin, 
         for (int i = j; i < Q; i += T) cp_async8(gs + c * Q + i, g + i);
     }
     cp_async_commit();
+    pdl_wait();   // the Ghat rows above are constant; the slab is pass 1's
     float2 v[CW][E];
 #pragma unroll
     for (int t = 0; t < E / 2; ++t) {
@@ -368,6 +387,7 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16(int nin, 
                 v[c][e * R + r] = v[c][e * R + r] * gs[c * Q + (kz <= P / 2 ? kz : P - kz)];
             }
     inv_stages<LP, LE, 0, false>(v, buf, j, tw);
+    pdl_trigger();
 #pragma unroll
     for (int t = 0; t < E; ++t) {
         const int z = j + t * T;
@@ -434,12 +454,12 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 // shortfall: bytes the barrier expects beyond what the boxes deliver (0; a test sets
 // it to make the wait run out with no copy left in flight).
 template <int LP, int LE, int MINB>
-__global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma(const __grid_constant__ CUtensorMap map,
+__global__ void __launch_bounds__(Geo<LP, LE, kTmaCta>::THREADS, MINB) k_cols16_tma(const __grid_constant__ CUtensorMap map,
                                                                            int n, float2* __restrict__ X,
                                                                            const float2* __restrict__ ghat,
                                                                            const float2* __restrict__ tw,
                                                                            unsigned shortfall) {
-    using Gm = Geo<LP, LE>;
+    using Gm = Geo<LP, LE, kTmaCta>;
     constexpr int CW = 2;
     using EL = float4;
     constexpr int P = Gm::P, T = Gm::T, E = Gm::E, R = 1 << Gm::LRL, Q = P / 2 + 1, G = Gm::G;
@@ -465,6 +485,14 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma(const
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
     __syncthreads();
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+        const int kx = kx0 + c;
+        const float2* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * Q;
+        for (int i = j; i < Q; i += T) cp_async8(gs + c * Q + i, g + i);
+    }
+    cp_async_commit();
+    pdl_wait();   // the Ghat rows above are constant; the slab is pass 1's
     if (threadIdx.x == 0) {
         const unsigned bytes = (unsigned)(G * nbox * BR * sizeof(EL)) + shortfall;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -475,13 +503,6 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma(const
             for (int k = 0; k < nbox; ++k) tma_load_2d(stg + k * BR, &map, x, k * BR, bar);
         }
     }
-#pragma unroll
-    for (int c = 0; c < CW; ++c) {
-        const int kx = kx0 + c;
-        const float2* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * Q;
-        for (int i = j; i < Q; i += T) cp_async8(gs + c * Q + i, g + i);
-    }
-    cp_async_commit();
     if (!mbar_wait(bar, 0)) atomicOr(&failed, 1);
     __syncthreads();
     if (failed) {  // rows of this CTA's tiles become NaN: visible to every residual check
@@ -511,6 +532,7 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma(const
                 v[c][e * R + r] = v[c][e * R + r] * gs[c * Q + (kz <= P / 2 ? kz : P - kz)];
             }
     inv_stages<LP, LE, 0, false>(v, buf, j, tw);
+    pdl_trigger();
     __syncthreads();  // every thread is done with the exchange buffer
 #pragma unroll
     for (int t = 0; t < E; ++t) {
@@ -535,12 +557,12 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma(const
 // transforms and summation order as the scalar form; the products are contracted
 // to fused multiply-adds in a fixed pattern (results agree to FP32 rounding).
 template <int LP, int LE, int MINB>
-__global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma2(const __grid_constant__ CUtensorMap map,
+__global__ void __launch_bounds__(Geo<LP, LE, kTmaCta>::THREADS, MINB) k_cols16_tma2(const __grid_constant__ CUtensorMap map,
                                                                             int n, float2* __restrict__ X,
                                                                             const float2* __restrict__ ghat,
                                                                             const float2* __restrict__ tw,
                                                                             unsigned shortfall) {
-    using Gm = Geo<LP, LE>;
+    using Gm = Geo<LP, LE, kTmaCta>;
     constexpr int CW = 2;
     using EL = typename Elem<1, CP>::T;
     constexpr int P = Gm::P, T = Gm::T, E = Gm::E, R = 1 << Gm::LRL, Q = P / 2 + 1, G = Gm::G;
@@ -567,6 +589,14 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma2(cons
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
     __syncthreads();
+#pragma unroll
+    for (int c = 0; c < CW; ++c) {
+        const int kx = kx0 + c;
+        const float2* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * Q;
+        for (int i = j; i < Q; i += T) cp_async8(gs + c * Q + i, g + i);
+    }
+    cp_async_commit();
+    pdl_wait();   // the Ghat rows above are constant; the slab is pass 1's
     if (threadIdx.x == 0) {
         const unsigned bytes = (unsigned)(G * nbox * BR * sizeof(EL)) + shortfall;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -577,13 +607,6 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma2(cons
             for (int k = 0; k < nbox; ++k) tma_load_2d(dst + k * BR, &map, x, k * BR, bar);
         }
     }
-#pragma unroll
-    for (int c = 0; c < CW; ++c) {
-        const int kx = kx0 + c;
-        const float2* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * Q;
-        for (int i = j; i < Q; i += T) cp_async8(gs + c * Q + i, g + i);
-    }
-    cp_async_commit();
     if (!mbar_wait(bar, 0)) atomicOr(&failed, 1);
     __syncthreads();
     if (failed) {
@@ -613,6 +636,7 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16_tma2(cons
             v[0][e * R + r] = cmul2(v[0][e * R + r], gs[kq], gs[Q + kq]);
         }
     inv_stages<LP, LE, 0, false>(v, buf, j, tw);
+    pdl_trigger();
     __syncthreads();
 #pragma unroll
     for (int t = 0; t < E; ++t) {
@@ -648,6 +672,7 @@ __global__ void __launch_bounds__(Geo<LP, 4>::THREADS, 4) k_rows16_inv(int nrows
     UIO* us = reinterpret_cast<UIO*>(buf);  // the row of u, once the exchanges are done
     const int z = blockIdx.x * Gm::G + grp;
     const bool live = z < nrows;
+    pdl_wait();
     float2 v[1][E];
     const float2* xr = X + (size_t)(live ? z : 0) * P;
 #pragma unroll
@@ -666,6 +691,7 @@ __global__ void __launch_bounds__(Geo<LP, 4>::THREADS, 4) k_rows16_inv(int nrows
         cp_async_commit();
     };
     inv_stages<LP, 4, 0, true>(v, buf, j, tw, prefetch_u);
+    pdl_trigger();
     cp_async_wait_all();  // this thread's own copies: no barrier needed
     if (!live) return;
 #pragma unroll
@@ -683,14 +709,14 @@ constexpr size_t rinv_smem() {  // the row of u (P/2 elements) reuses the exchan
     static_assert(sizeof(UIO) * (Gm::P / 2) <= sizeof(float2) * Gm::SLOTS, "u row must fit");
     return sizeof(float2) * Gm::G * Gm::SLOTS;
 }
-template <int LP, int LE, int CW>
+template <int LP, int LE, int CW, int MINT = kSmallCta>
 constexpr size_t cols_smem() {
-    using Gm = Geo<LP, LE>;
+    using Gm = Geo<LP, LE, MINT>;
     return sizeof(float2) * CW * Gm::G * Gm::SLOTS + sizeof(float2) * Gm::G * CW * (Gm::P / 2 + 1);
 }
 template <int LP, int LE>
 constexpr size_t cols_tma_smem() {
-    return cols_smem<LP, LE, 2>() + 16;  // + the mbarrier and the CTA's failure flag
+    return cols_smem<LP, LE, 2, kTmaCta>() + 16;  // + the mbarrier and the CTA's failure flag
 }
 template <int LP>
 constexpr size_t row_smem16() {
@@ -699,14 +725,13 @@ constexpr size_t row_smem16() {
 
 // Column-pass tile shapes (ls_handle::fft_variant): 0 = radix 16, 1 column, 3 CTAs/SM;
 // 2 = radix 16, 2 columns, 2 CTAs/SM; 3 = radix 16, 1 column, 2 CTAs/SM;
-// 4 = radix 8, 1 column, 2 CTAs/SM (of up to 512 threads); 5 = radix 8, 2 columns, 1 CTA/SM;
+// 4 = radix 8, 1 column, 2 CTAs/SM (of up to 512 threads; the one that P < 256 has); 5 = radix 8, 2 columns, 1 CTA/SM;
 // 6, 7 = shapes 2, 5 with the tiles moved by TMA; 8 = shape 6 in packed FP32x2 arithmetic.
 template <int LP, int LE, int CW, int MINB>
 int cols_launch(ls_handle* h, int n, float2* X, const float2* gh, const float2* tw) {
     using Gm = Geo<LP, LE>;
-    LS_LAUNCH(h, (k_cols16<LP, LE, CW, MINB>), (unsigned)(Gm::P / CW / Gm::G), Gm::THREADS,
-              (cols_smem<LP, LE, CW>()), n, n, X, gh, tw);
-    return LS_OK;
+    return ls_launch_pdl(h, k_cols16<LP, LE, CW, MINB>, dim3((unsigned)(Gm::P / CW / Gm::G)), dim3(Gm::THREADS),
+                         cols_smem<LP, LE, CW>(), n, n, X, gh, tw);
 }
 
 // Tensor map of the n x P slab for the TMA shapes: FP32 elements, rows of 2P, boxes
@@ -727,7 +752,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 template <int LP, int LE, int MINB, bool PACKED = false>
 int cols_launch_tma(ls_handle* h, int n, float2* X, const float2* gh, const float2* tw) {
-    using Gm = Geo<LP, LE>;
+    using Gm = Geo<LP, LE, kTmaCta>;
     constexpr int P = Gm::P, BR = P / 2 < 256 ? P / 2 : 256;
     auto enc = tensor_map_encoder();
     if (!enc) return LS_ECUDA;
@@ -740,13 +765,9 @@ int cols_launch_tma(ls_handle* h, int n, float2* X, const float2* gh, const floa
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return LS_ECUDA;
-    if constexpr (PACKED)
-        LS_LAUNCH(h, (k_cols16_tma2<LP, LE, MINB>), (unsigned)(P / 2 / Gm::G), Gm::THREADS, (cols_tma_smem<LP, LE>()),
-                  map, n, X, gh, tw, g_tma_shortfall);
-    else
-        LS_LAUNCH(h, (k_cols16_tma<LP, LE, MINB>), (unsigned)(P / 2 / Gm::G), Gm::THREADS, (cols_tma_smem<LP, LE>()),
-                  map, n, X, gh, tw, g_tma_shortfall);
-    return LS_OK;
+    return ls_launch_pdl(h, PACKED ? k_cols16_tma2<LP, LE, MINB> : k_cols16_tma<LP, LE, MINB>,
+                         dim3((unsigned)(P / 2 / Gm::G)), dim3(Gm::THREADS), cols_tma_smem<LP, LE>(), map, n, X, gh, tw,
+                         g_tma_shortfall);
 }
 
 template <int LP, typename UIO>
@@ -757,8 +778,10 @@ int apply_lp(ls_handle* h, const UIO* u, UIO* y, float2* X, int shape) {
     const float2* gh = static_cast<const float2*>(h->ghat32);
     const unsigned rows_grid = (unsigned)((n + Gm::G - 1) / Gm::G);
     SrcMU<float, UIO> src{h->m32, u, n};
-    LS_LAUNCH(h, (k_rows16_fwd<LP, SrcMU<float, UIO>>), rows_grid, Gm::THREADS, row_smem16<LP>(), n, n, src, X, tw);
-    switch (shape) {
+    LS_TRY(ls_launch_pdl(h, k_rows16_fwd<LP, SrcMU<float, UIO>>, dim3(rows_grid), dim3(Gm::THREADS), row_smem16<LP>(), n,
+                         n, src, X, tw));
+    if constexpr (LP < 8) LS_TRY((cols_launch<LP, 3, 1, 2>(h, n, X, gh, tw)));
+    else switch (shape) {
         case 2: LS_TRY((cols_launch<LP, 4, 2, 2>(h, n, X, gh, tw))); break;
         case 3: LS_TRY((cols_launch<LP, 4, 1, 2>(h, n, X, gh, tw))); break;
         case 4: LS_TRY((cols_launch<LP, 3, 1, 2>(h, n, X, gh, tw))); break;
@@ -768,14 +791,17 @@ int apply_lp(ls_handle* h, const UIO* u, UIO* y, float2* X, int shape) {
         case 8: LS_TRY((cols_launch_tma<LP, 4, 2, true>(h, n, X, gh, tw))); break;
         default: LS_TRY((cols_launch<LP, 4, 1, 3>(h, n, X, gh, tw))); break;
     }
-    LS_LAUNCH(h, (k_rows16_inv<LP, UIO>), rows_grid, Gm::THREADS, (rinv_smem<LP, UIO>()), n, n, X, u, y, tw);
-    return LS_OK;
+    return ls_launch_pdl(h, k_rows16_inv<LP, UIO>, dim3(rows_grid), dim3(Gm::THREADS), rinv_smem<LP, UIO>(), n, n,
+                         static_cast<const float2*>(X), u, y, tw);
 }
 
 template <typename UIO>
 int apply_any(ls_handle* h, const UIO* u, UIO* y, int shape) {
     float2* X = static_cast<float2*>(h->fftws);
     switch (h->lp) {
+        case 5: return apply_lp<5>(h, u, y, X, shape);
+        case 6: return apply_lp<6>(h, u, y, X, shape);
+        case 7: return apply_lp<7>(h, u, y, X, shape);
         case 8: return apply_lp<8>(h, u, y, X, shape);
         case 9: return apply_lp<9>(h, u, y, X, shape);
         case 10: return apply_lp<10>(h, u, y, X, shape);
@@ -807,10 +833,18 @@ int optin_lp() {
 
 }  // namespace
 
-bool ls_fft16_supported(const ls_handle* h) { return h->lp >= 8 && h->lp <= 12; }
+// shape 4 takes 32 <= P <= 4096, the others (but 1, the generic path) 256 <= P <= 4096
+bool ls_fft16_supported(const ls_handle* h, int shape) {
+    return shape != 1 && h->lp >= (shape == 4 ? 5 : 8) && h->lp <= 12;
+}
+
+// The shape a handle starts with: radix-8 1-column tiles up to P = 512 (n = 128: 9.1 us on the
+// device against 11.4 with 2-column radix-16 tiles, 256: 10.3 against 15.4), TMA tiles in
+// packed FP32x2 arithmetic above (512: 16.0 against 16.4, 1024: 43.3 against 51.7, 2048: 139
+// against 191).
+int ls_fft16_default(const ls_handle* h) { return h->lp <= 9 ? 4 : 8; }
 
 int ls_fft16_init(ls_handle* h) {
-    if (!ls_fft16_supported(h)) return LS_OK;
     LS_TRY(optin_lp<8>());
     LS_TRY(optin_lp<9>());
     LS_TRY(optin_lp<10>());

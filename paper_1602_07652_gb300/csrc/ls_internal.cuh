@@ -271,7 +271,7 @@ struct ls_handle {
     int learned_steps = 0;
 
     // choices of the autotuner (ls_tune.cu); defaults until ls_autotune runs
-    int fft_variant = 2;       // column-pass shape (256 <= P <= 4096): radix 16 with 0 = 1-column tiles,
+    int fft_variant = 2;       // column-pass shape (ls_fft16_default): radix 16 with 0 = 1-column tiles,
                                // 3 CTAs/SM; 2 = 2-column tiles; 3 = 1-column tiles, 2 CTAs/SM; radix 8 with
                                // 4 = 1-column tiles; 5 = 2-column tiles.  1: generic radix-8 4-column tiles
     static constexpr int kFftVariants = 9;
@@ -358,7 +358,8 @@ int ls_apply_mx(ls_handle* h, const double2* u, double2* y);    // FP64 I/O, FP3
 int ls_apply_df(ls_handle* h, const double2* u, double2* y);    // FP64 I/O, double-float arithmetic
 int ls_rhs_df(ls_handle* h, double theta, double2* f);          // incident right-hand side, double-float
 int ls_rhs(ls_handle* h, double theta, double2* f);             // ls_rhs_df if h->dfloat, else ls_rhs64
-bool ls_fft16_supported(const ls_handle* h);                     // radix-16 FP32 path: 256 <= P <= 4096
+bool ls_fft16_supported(const ls_handle* h, int shape);          // fft_variant on the specialised FP32 path
+int ls_fft16_default(const ls_handle* h);
 int ls_fft16_init(ls_handle* h);
 int ls_apply32_fft16(ls_handle* h, const float2* u, float2* y, int shape);  // shape: fft_variant != 1
 int ls_apply_mx_fft16(ls_handle* h, const double2* u, double2* y, int shape);

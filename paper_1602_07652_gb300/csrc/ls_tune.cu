@@ -61,7 +61,7 @@ extern "C" int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out) {
         float best = 0;
         int pick = 0;
         for (int v = 0; v < ls_handle::kFftVariants && rc == LS_OK; ++v) {
-            if (v != 1 && !ls_fft16_supported(h)) {
+            if (v != 1 && !ls_fft16_supported(h, v)) {
                 t.fft_ms[v] = -1;
                 continue;
             }
