@@ -101,4 +101,35 @@ template <> __device__ __forceinline__ cdfl ldg_c<cdfl>(const cdfl* p) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(p));
     return cdfl{dfl(v.x, v.y), dfl(v.z, v.w)};
 }
+
+// m u_I in double-float: the incident wave's factors and the medium as double-float tables
+struct SrcIncDf {
+    const dfl* m;
+    const cdfl* ex;
+    const cdfl* ez;
+    int n;
+    template <typename C>
+    __device__ __forceinline__ cdfl load(int z, int x) const {
+        return m[(size_t)z * n + x] * (ldg_c(&ex[x]) * ldg_c(&ez[z]));
+    }
+};
+
+// d * exp(-DIR 2 pi i idx / 16) (the in-register DFT's constant rotations, found by argument-
+// dependent lookup): the odd multiples of pi/4 as one sum and one product per component (18
+// operations instead of 25), the others as one two-term product sum (20).
+__device__ __forceinline__ dfl df_cos16(int i) {   // cos(2 pi i / 16), i in [0, 8]
+    return i == 1 ? dfl(0.92387953251128675613) : i == 3 ? dfl(0.38268343236508977173)
+         : i == 5 ? dfl(-0.38268343236508977173) : i == 7 ? dfl(-0.92387953251128675613) : dfl(0.f, 0.f);
+}
+template <int DIR>
+__device__ __forceinline__ cdfl rot16(cdfl d, int idx) {
+    const dfl h(0.70710678118654752440);
+    if (idx == 0) return d;
+    if (idx == 4) return DIR > 0 ? cdfl{d.y, -d.x} : cdfl{-d.y, d.x};
+    if (idx == 2) return DIR > 0 ? cdfl{(d.x + d.y) * h, (d.y - d.x) * h} : cdfl{(d.x - d.y) * h, (d.x + d.y) * h};
+    if (idx == 6) return DIR > 0 ? cdfl{(d.y - d.x) * h, -((d.x + d.y) * h)} : cdfl{-((d.x + d.y) * h), (d.x - d.y) * h};
+    const dfl c = df_cos16(idx), s = df_cos16(idx <= 4 ? 4 - idx : idx - 4);
+    if (DIR > 0) return cdfl{df_dot2(d.x, c, d.y, s), df_dot2(d.y, c, -d.x, s)};
+    return cdfl{df_dot2(d.x, c, -d.y, s), df_dot2(d.y, c, d.x, s)};
+}
 #endif

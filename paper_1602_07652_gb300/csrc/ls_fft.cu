@@ -409,18 +409,6 @@ __global__ void k_incident_factors_df(int n, double wh, double cth, double sth, 
     ez[i] = ccast<cdfl>(make_double2(c, s));
 }
 
-// m u_I in double-float: the incident wave's factors and the medium as double-float tables
-struct SrcIncDf {
-    const dfl* m;
-    const cdfl* ex;
-    const cdfl* ez;
-    int n;
-    template <typename C>
-    __device__ __forceinline__ cdfl load(int z, int x) const {
-        return m[(size_t)z * n + x] * (ldg_c(&ex[x]) * ldg_c(&ez[z]));
-    }
-};
-
 __global__ void k_quad_to32(size_t cnt, const double2* a, float2* b) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < cnt) b[i] = ccast<float2>(a[i]);
@@ -499,6 +487,10 @@ int ls_fft_init(ls_handle* h) {
     LS_TRY(allow_smem(k_rows_fwd<float, E32, SrcMU<float, double2>>, row_smem32(P)));
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<float2>>, row_smem32(P)));
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<double2>>, row_smem32(P)));
+    if (h->lp >= 6) {
+        LS_TRY(ls_wide64_init());
+        LS_TRY(ls_widedf_init());
+    }
     h->fft_variant = ls_fft16_default(h);
     return ls_fft16_init(h);
 }
@@ -539,6 +531,7 @@ int ls_spectrum_build(ls_handle* h, const double2* gtab) {
 }
 
 int ls_apply64(ls_handle* h, const double2* u, double2* y) {
+    if (h->lp >= 6) return ls_wide64_apply(h, u, y);
     const int n = h->n, P = h->P;
     const FftPlan& pl = h->plan64;
     double2* X = static_cast<double2*>(h->fftws);
@@ -553,9 +546,11 @@ int ls_apply64(ls_handle* h, const double2* u, double2* y) {
     return LS_OK;
 }
 
+// (P >= 64 has passes of its own, here and below: ls_fft_wide.cuh)
 // The FP64 apply's three passes in double-float arithmetic (ls_dfloat.cuh): FP64 I/O,
 // about 48 significant bits inside, on the FP32 pipes.
 int ls_apply_df(ls_handle* h, const double2* u, double2* y) {
+    if (h->lp >= 6) return ls_widedf_apply(h, u, y);
     const int n = h->n, P = h->P;
     const FftPlan& pl = h->plan64;
     cdfl* X = static_cast<cdfl*>(h->fftws);
@@ -606,6 +601,7 @@ int ls_rhs64(ls_handle* h, double theta, double2* f) {
     double2* X = static_cast<double2*>(h->fftws);
     LS_LAUNCH(h, k_incident_factors, (n + 255) / 256, 256, 0, n, h->omega * h->h, std::cos(theta),
               std::sin(theta), h->incx, h->incz);
+    if (h->lp >= 6) return ls_wide64_rhs(h, f);
     SrcInc<double> src{h->m64, h->incx, h->incz, n};
     LS_LAUNCH(h, (k_rows_fwd<double, E64, SrcInc<double>>), n, P / E64, row_smem64(P),
               pl, n, src, X, h->tw64);
@@ -623,6 +619,7 @@ int ls_rhs_df(ls_handle* h, double theta, double2* f) {
     cdfl* X = static_cast<cdfl*>(h->fftws);
     LS_LAUNCH(h, k_incident_factors_df, (n + 255) / 256, 256, 0, n, h->omega * h->h, std::cos(theta),
               std::sin(theta), h->incxdf, h->inczdf);
+    if (h->lp >= 6) return ls_widedf_rhs(h, f);
     SrcIncDf src{h->mdf, h->incxdf, h->inczdf, n};
     LS_LAUNCH(h, (k_rows_fwd<dfl, E64, SrcIncDf>), n, P / E64, row_smem64(P), pl, n, src, X, h->twdf);
     LS_LAUNCH(h, (k_cols_vec<dfl, EV, CW64, 0>), P / CW64, (P / EV), col_smem(P), h->planc64, n, n, X, h->ghatdf,

@@ -361,6 +361,13 @@ int ls_rhs(ls_handle* h, double theta, double2* f);             // ls_rhs_df if 
 bool ls_fft16_supported(const ls_handle* h, int shape);          // fft_variant on the specialised FP32 path
 int ls_fft16_default(const ls_handle* h);
 int ls_fft16_init(ls_handle* h);
+// FP64 and double-float passes specialised on P >= 64 (ls_fft_wide64.cu, ls_fft_widedf.cu)
+int ls_wide64_init();
+int ls_wide64_apply(ls_handle* h, const double2* u, double2* y);
+int ls_wide64_rhs(ls_handle* h, double2* f);
+int ls_widedf_init();
+int ls_widedf_apply(ls_handle* h, const double2* u, double2* y);
+int ls_widedf_rhs(ls_handle* h, double2* f);
 int ls_apply32_fft16(ls_handle* h, const float2* u, float2* y, int shape);  // shape: fft_variant != 1
 int ls_apply_mx_fft16(ls_handle* h, const double2* u, double2* y, int shape);
 int ls_rhs64(ls_handle* h, double theta, double2* f);           // f = -w^2 G (m u_I)

@@ -45,3 +45,31 @@ def test_fp32_apply_at_the_edges_of_each_length(n):
         err = np.linalg.norm(y.cpu().numpy() - ref) / np.linalg.norm(ref)
         assert err < tol, (shape, err)
     s.close()
+
+
+@pytest.mark.parametrize("n", [16, 17, 32, 33, 63, 64, 65, 129, 256, 257, 513])
+def test_fp64_and_double_float_applies_at_the_edges_of_each_length(n):
+    # P = 64 .. 2048 have kernels of their own (P = 32: the generic ones); two applies in a
+    # row in place, and the incident right-hand side.  Bounds: FP64 FFT rounding and the
+    # double-float format's 2^-46 against the FP64 result, with a factor of 10 each; the
+    # kernel weights' own rounding against the oracle.
+    w = inputs.omega_for_ppw(n, 10.24)
+    m = inputs.bump_medium(n, nbumps=5, seed=n)
+    L = next(d for d in range(1, n + 1) if n % d == 0 and n // d + 4 <= 112)
+    s = binding.Solver(torch.from_numpy(m), w, layers=L, ext=2, precision=binding.LS_MIXED)
+    u = inputs.random_field(n, n)
+    ref = greens.apply_H(greens.apply_H(u, m, 1.0 / n, w), m, 1.0 / n, w)
+    out = {}
+    for name, fn in (("fp64", s.ls_apply), ("df", s.ls_apply_double_float)):
+        y = torch.from_numpy(u).cuda()
+        fn(y, y)
+        fn(y, y)
+        out[name] = y.cpu().numpy()
+        assert np.linalg.norm(out[name] - ref) / np.linalg.norm(ref) < 1e-11, name
+    assert np.linalg.norm(out["df"] - out["fp64"]) / np.linalg.norm(ref) < 10 * 2 * math.log2(2 * n) * 2.0 ** -46
+    f = greens.rhs(m, 1.0 / n, w, greens.incident_plane_wave(n, w, 0.3))
+    for df in (1, 0):
+        s.ls_set_double_float(df)
+        g = s.ls_incident_rhs(0.3).cpu().numpy()
+        assert np.linalg.norm(g - f) / np.linalg.norm(f) < 1e-11, df
+    s.close()
