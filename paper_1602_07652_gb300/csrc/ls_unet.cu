@@ -339,42 +339,93 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_wgrad(WgradArgs a) {
     }
 }
 
-// db[c] += sum over a pixel chunk of dy[p][c]
-__global__ void k_bias_grad(const bf16* __restrict__ dy, int ds, int dof, int cout, int M, int chunk,
-                            float* __restrict__ db) {
-    const int c = threadIdx.x;
-    if (c >= cout) return;
+// Eight consecutive channels of a pixel: channel counts, strides and offsets are multiples of
+// 16, so every elementwise kernel moves them in one 16-byte access (one channel per thread ran
+// at a fifth of the memory rate).
+struct Ch8 {
+    float v[8];
+};
+__device__ __forceinline__ Ch8 ld8(const bf16* p) {
+    const uint4 u = *reinterpret_cast<const uint4*>(p);
+    const unsigned w[4] = {u.x, u.y, u.z, u.w};
+    Ch8 o;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o.v[2 * i] = __uint_as_float(w[i] << 16);
+        o.v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+    return o;
+}
+__device__ __forceinline__ void st8(bf16* p, const Ch8& a) {
+    __align__(16) bf16 o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o[i] = __float2bfloat16(a.v[i]);
+    *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(o);
+}
+
+// db[c] += sum over a pixel chunk of dy[p][c].  256 threads: thread (lane, g) takes channels
+// 8 g .. 8 g + 7 of pixels lane, lane + lanes, ...; the lanes' sums meet in shared memory.
+// (One thread per channel took 40 us a layer, 1024 loads one after the other.)
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, int ds, int dof, int cout, int M,
+                                                   int chunk, float* __restrict__ db) {
+    __shared__ float red[256][9];
     const int pbeg = blockIdx.x * chunk, pend = min(M, pbeg + chunk);
-    float s = 0.0f;
-    for (int p = pbeg; p < pend; ++p) s += __bfloat162float(dy[(size_t)p * ds + dof + c]);
-    atomicAdd(&db[c], s);
+    for (int g0 = 0; g0 < cout / 8; g0 += 256) {
+        const int ng = min(cout / 8 - g0, 256), lanes = 256 / ng;
+        const int lane = threadIdx.x / ng, g = threadIdx.x - lane * ng;
+        float s[8] = {};
+        if (lane < lanes)
+            for (int p = pbeg + lane; p < pend; p += lanes) {
+                const Ch8 v = ld8(dy + (size_t)p * ds + dof + 8 * (g0 + g));
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s[i] += v.v[i];
+            }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) red[threadIdx.x][i] = s[i];
+        __syncthreads();
+        for (int c = threadIdx.x; c < 8 * ng; c += 256) {
+            float t = 0.0f;
+            for (int l = 0; l < lanes; ++l) t += red[l * ng + (c >> 3)][c & 7];
+            atomicAdd(&db[8 * g0 + c], t);
+        }
+        __syncthreads();
+    }
 }
 
 // out = (y > 0) ? g : 0 on matching views (out dense, c channels)
 __global__ void k_relu_mask(size_t M, int c, const bf16* __restrict__ g, int gs, int go, const bf16* __restrict__ y,
                             int ys, int yo, bf16* __restrict__ out) {
-    const size_t n = M * c;
+    const int c8 = c / 8;
+    const size_t n = M * c8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t p = i / c;
-        const int k = (int)(i % c);
-        const float yv = __bfloat162float(y[p * ys + yo + k]);
-        out[i] = yv > 0.0f ? g[p * gs + go + k] : __float2bfloat16(0.0f);
+        const size_t p = i / c8;
+        const int k = 8 * (int)(i % c8);
+        const Ch8 yv = ld8(y + p * ys + yo + k);
+        Ch8 gv = ld8(g + p * gs + go + k);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) gv.v[e] = yv.v[e] > 0.0f ? gv.v[e] : 0.0f;
+        st8(out + 8 * i, gv);
     }
 }
 
 // 2x2 average pool: in (nb, H, W) view -> out dense (nb, H/2, W/2, c)
 __global__ void k_pool(int nb, int H, int W, int c, const bf16* __restrict__ x, int xs, int xo, bf16* __restrict__ y) {
-    const int H2 = H / 2, W2 = W / 2;
-    const size_t n = (size_t)nb * H2 * W2 * c;
+    const int H2 = H / 2, W2 = W / 2, c8 = c / 8;
+    const size_t n = (size_t)nb * H2 * W2 * c8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i % c);
-        const size_t q = i / c;
+        const int k = 8 * (int)(i % c8);
+        const size_t q = i / c8;
         const int xx = (int)(q % W2), yy = (int)((q / W2) % H2), b = (int)(q / ((size_t)W2 * H2));
-        float s = 0.0f;
+        Ch8 s{};
         for (int dy = 0; dy < 2; ++dy)
-            for (int dx = 0; dx < 2; ++dx)
-                s += __bfloat162float(x[((size_t)b * H * W + (size_t)(2 * yy + dy) * W + 2 * xx + dx) * xs + xo + k]);
-        y[i] = __float2bfloat16(0.25f * s);
+            for (int dx = 0; dx < 2; ++dx) {
+                const Ch8 v = ld8(x + ((size_t)b * H * W + (size_t)(2 * yy + dy) * W + 2 * xx + dx) * xs + xo + k);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) s.v[e] += v.v[e];
+            }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s.v[e] *= 0.25f;
+        st8(y + 8 * i, s);
     }
 }
 
@@ -382,43 +433,54 @@ __global__ void k_pool(int nb, int H, int W, int c, const bf16* __restrict__ x, 
 // skip view + g2[p / 2] / 4
 __global__ void k_pool_bwd_add(int nb, int H, int W, int c, const bf16* __restrict__ g2, const bf16* __restrict__ sk,
                                int ss, int so, bf16* __restrict__ out) {
-    const size_t n = (size_t)nb * H * W * c;
+    const int c8 = c / 8;
+    const size_t n = (size_t)nb * H * W * c8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i % c);
-        const size_t q = i / c;
+        const int k = 8 * (int)(i % c8);
+        const size_t q = i / c8;
         const int xx = (int)(q % W), yy = (int)((q / W) % H), b = (int)(q / ((size_t)W * H));
         const size_t q2 = (size_t)b * (H / 2) * (W / 2) + (size_t)(yy / 2) * (W / 2) + xx / 2;
-        float v = 0.25f * __bfloat162float(g2[q2 * c + k]);
-        if (sk) v += __bfloat162float(sk[q * ss + so + k]);
-        out[i] = __float2bfloat16(v);
+        Ch8 v = ld8(g2 + q2 * c + k);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v.v[e] *= 0.25f;
+        if (sk) {
+            const Ch8 t = ld8(sk + q * ss + so + k);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v.v[e] += t.v[e];
+        }
+        st8(out + 8 * i, v);
     }
 }
 
 // nearest 2x upsampling: in (nb, H/2, W/2) view -> out dense (nb, H, W, c)
 __global__ void k_up(int nb, int H, int W, int c, const bf16* __restrict__ x, int xs, int xo, bf16* __restrict__ y) {
-    const size_t n = (size_t)nb * H * W * c;
+    const int c8 = c / 8;
+    const size_t n = (size_t)nb * H * W * c8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i % c);
-        const size_t q = i / c;
+        const int k = 8 * (int)(i % c8);
+        const size_t q = i / c8;
         const int xx = (int)(q % W), yy = (int)((q / W) % H), b = (int)(q / ((size_t)W * H));
         const size_t q2 = (size_t)b * (H / 2) * (W / 2) + (size_t)(yy / 2) * (W / 2) + xx / 2;
-        y[i] = x[q2 * xs + xo + k];
+        *reinterpret_cast<uint4*>(y + 8 * i) = *reinterpret_cast<const uint4*>(x + q2 * xs + xo + k);
     }
 }
 
 // gradient of the upsampling: out (nb, H/2, W/2, c) dense = sum of the 4 children of g (dense, H x W)
 __global__ void k_up_bwd(int nb, int H, int W, int c, const bf16* __restrict__ g, bf16* __restrict__ out) {
-    const int H2 = H / 2, W2 = W / 2;
-    const size_t n = (size_t)nb * H2 * W2 * c;
+    const int H2 = H / 2, W2 = W / 2, c8 = c / 8;
+    const size_t n = (size_t)nb * H2 * W2 * c8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i % c);
-        const size_t q = i / c;
+        const int k = 8 * (int)(i % c8);
+        const size_t q = i / c8;
         const int xx = (int)(q % W2), yy = (int)((q / W2) % H2), b = (int)(q / ((size_t)W2 * H2));
-        float s = 0.0f;
+        Ch8 s{};
         for (int dy = 0; dy < 2; ++dy)
-            for (int dx = 0; dx < 2; ++dx)
-                s += __bfloat162float(g[((size_t)b * H * W + (size_t)(2 * yy + dy) * W + 2 * xx + dx) * c + k]);
-        out[i] = __float2bfloat16(s);
+            for (int dx = 0; dx < 2; ++dx) {
+                const Ch8 v = ld8(g + ((size_t)b * H * W + (size_t)(2 * yy + dy) * W + 2 * xx + dx) * c + k);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) s.v[e] += v.v[e];
+            }
+        st8(out + 8 * i, s);
     }
 }
 
@@ -631,21 +693,26 @@ int wgrad(ls_net* n, int li, const bf16* dy, View x, int H, int W, int M) {
     a.x = x.p; a.xs = x.stride; a.xo = x.off; a.cin = Ly.cin;
     a.dw = n->g + Ly.woff;
     a.H = H; a.W = W; a.M = M;
-    a.chunk = 4096;
     const int BM = Ly.cout >= 64 ? 64 : Ly.cout;
     const int K9 = 9 * Ly.cin;
+    // pixels per CTA: a CTA runs through its chunk 32 pixels at a time, 2 us each, so chunks are
+    // short enough for about 16 CTAs per SM (a chunk of 4096 took 220 to 280 us a layer
+    // whatever its size), and long enough that their atomic sums stay few
+    const int tiles = ((K9 + 63) / 64) * (Ly.cout / BM);
+    a.chunk = (int)((size_t)M * tiles / (152 * 16) + 31) / 32 * 32;
+    a.chunk = a.chunk < 256 ? 256 : (a.chunk > 4096 ? 4096 : a.chunk);
     const dim3 grid((unsigned)((K9 + 63) / 64), (unsigned)(Ly.cout / BM), (unsigned)((M + a.chunk - 1) / a.chunk));
     if (BM == 64) NET_LAUNCH(n, k_conv_wgrad<64>, grid, kConvThreads, 0, a);
     else if (BM == 32) NET_LAUNCH(n, k_conv_wgrad<32>, grid, kConvThreads, 0, a);
     else NET_LAUNCH(n, k_conv_wgrad<16>, grid, kConvThreads, 0, a);
     const int bchunk = 1024;
-    NET_LAUNCH(n, k_bias_grad, (unsigned)((M + bchunk - 1) / bchunk), Ly.cout, 0, dy, Ly.cout, 0, Ly.cout, M, bchunk,
+    NET_LAUNCH(n, k_bias_grad, (unsigned)((M + bchunk - 1) / bchunk), 256, 0, dy, Ly.cout, 0, Ly.cout, M, bchunk,
                n->g + Ly.boff);
     return LS_OK;
 }
 
 int mask(ls_net* n, size_t M, int c, View g, View y) {
-    NET_LAUNCH(n, k_relu_mask, grid_for(M * c), 256, 0, M, c, g.p, g.stride, g.off, y.p, y.stride, y.off, n->tmp);
+    NET_LAUNCH(n, k_relu_mask, grid_for(M * c / 8), 256, 0, M, c, g.p, g.stride, g.off, y.p, y.stride, y.off, n->tmp);
     return LS_OK;
 }
 
@@ -672,7 +739,7 @@ int forward(ls_net* n, int nb, int H, int W, const double2* r, const double* m) 
     for (int l = 0; l < n->L; ++l) {
         const int Hl = H >> l, Wl = W >> l, M = nb * Hl * Wl, c = n->ch(l);
         if (l > 0) {
-            NET_LAUNCH(n, k_pool, grid_for((size_t)M * h.c), 256, 0, nb, 2 * Hl, 2 * Wl, h.c, h.p, h.stride, h.off,
+            NET_LAUNCH(n, k_pool, grid_for((size_t)M * h.c / 8), 256, 0, nb, 2 * Hl, 2 * Wl, h.c, h.p, h.stride, h.off,
                        n->pool[l]);
             h = View{n->pool[l], h.c, 0, h.c};
         }
@@ -684,7 +751,7 @@ int forward(ls_net* n, int nb, int H, int W, const double2* r, const double* m) 
     }
     for (int l = n->L - 2; l >= 0; --l) {
         const int Hl = H >> l, Wl = W >> l, M = nb * Hl * Wl, c = n->ch(l);
-        NET_LAUNCH(n, k_up, grid_for((size_t)M * h.c), 256, 0, nb, Hl, Wl, h.c, h.p, h.stride, h.off, n->up[l]);
+        NET_LAUNCH(n, k_up, grid_for((size_t)M * h.c / 8), 256, 0, nb, Hl, Wl, h.c, h.p, h.stride, h.off, n->up[l]);
         View up{n->up[l], 2 * c, 0, 2 * c};
         LS_TRY(conv(n, li_dec(n, l, 0), up, View{n->cat[l], 2 * c, 0, c}, Hl, Wl, M, true, false));
         LS_TRY(conv(n, li_dec(n, l, 1), View{n->cat[l], 2 * c, 0, 2 * c}, View{n->da[l], c, 0, c}, Hl, Wl, M, true,
@@ -719,14 +786,14 @@ int backward(ls_net* n, int nb, int H, int W) {
                     true));
         // through the upsampling into the output of level l + 1
         bf16* dst = l + 1 <= L - 2 ? n->g_dbo[l + 1] : n->g_bott;
-        NET_LAUNCH(n, k_up_bwd, grid_for((size_t)(M / 4) * 2 * c), 256, 0, nb, Hl, Wl, 2 * c, n->g_up[l], dst);
+        NET_LAUNCH(n, k_up_bwd, grid_for((size_t)(M / 4) * 2 * c / 8), 256, 0, nb, Hl, Wl, 2 * c, n->g_up[l], dst);
     }
     for (int l = L - 1; l >= 0; --l) {
         const int Hl = H >> l, Wl = W >> l, M = nb * Hl * Wl, c = n->ch(l);
         View out = l < L - 1 ? View{n->cat[l], 2 * c, c, c} : View{n->bott, c, 0, c};
         bf16* gout = n->g_bott;
         if (l < L - 1) {  // skip gradient + the gradient through the pool of level l + 1
-            NET_LAUNCH(n, k_pool_bwd_add, grid_for((size_t)M * c), 256, 0, nb, Hl, Wl, c, n->g_pool[l + 1],
+            NET_LAUNCH(n, k_pool_bwd_add, grid_for((size_t)M * c / 8), 256, 0, nb, Hl, Wl, c, n->g_pool[l + 1],
                        n->g_cat[l], 2 * c, c, n->g_eb[l]);
             gout = n->g_eb[l];
         }
