@@ -191,6 +191,63 @@ struct GemmTask {
     double a1, a2;  // real scalars (the reductions only need -1, +1)
 };
 
+// The same with the whole width of a matrix per CTA, for launches of many tasks: thread (g, c)
+// of 256 takes column c = tid % q and rows r0 + g, r0 + g + CG, ... (CG = 256 / q groups, RT
+// rows a thread), so that nearly every lane of the FP64 pipe works (q = 84: 252 of 256 lanes,
+// 4 chunks of 21 rows; 32 x 32 tiles kept 77 per cent of them busy).  A's entries are read
+// by broadcast, B's by consecutive lanes.
+template <int RT>
+__global__ void __launch_bounds__(256) k_gemm_wide(const GemmTask* __restrict__ tasks, int q) {
+    extern __shared__ __align__(16) double2 smw[];   // A: [16][CG * RT], B: [16][q]
+    const GemmTask tk = tasks[blockIdx.x];
+    const int CG = 256 / q, rows = CG * RT, r0 = blockIdx.y * rows;
+    const int g = threadIdx.x / q, c = threadIdx.x - g * q;
+    const bool act = g < CG;
+    double2* As = smw;
+    double2* Bs = smw + 16 * rows;
+    double2 acc[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+        const int r = r0 + g + CG * i;
+        acc[i] = (tk.C0 && act && r < q) ? tk.C0[c * q + r] : make_double2(0, 0);
+    }
+    for (int term = 0; term < 2; ++term) {
+        const double2* A = term == 0 ? tk.A1 : tk.A2;
+        const double2* B = term == 0 ? tk.B1 : tk.B2;
+        const double al = term == 0 ? tk.a1 : tk.a2;
+        if (!A) continue;
+        double2 part[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) part[i] = make_double2(0, 0);
+        for (int k0 = 0; k0 < q; k0 += 16) {
+            const int kn = q - k0 < 16 ? q - k0 : 16;
+            for (int e = threadIdx.x; e < kn * rows; e += 256) {
+                const int kk = e / rows, rr = e - kk * rows;
+                As[e] = r0 + rr < q ? A[(k0 + kk) * q + r0 + rr] : make_double2(0, 0);
+            }
+            for (int e = threadIdx.x; e < kn * q; e += 256) {   // Bs[kk][cc], read along k
+                const int cc = e / kn, kk = e - cc * kn;
+                Bs[kk * q + cc] = B[cc * q + k0 + kk];
+            }
+            __syncthreads();
+            if (act)
+                for (int kk = 0; kk < kn; ++kk) {
+                    const double2 b = Bs[kk * q + c];
+#pragma unroll
+                    for (int i = 0; i < RT; ++i) part[i] = cfma(As[kk * rows + g + CG * i], b, part[i]);
+                }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i) acc[i] = acc[i] + al * part[i];
+    }
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+        const int r = r0 + g + CG * i;
+        if (act && r < q) tk.C[c * q + r] = acc[i];
+    }
+}
+
 __global__ void __launch_bounds__(256) k_gemm(const GemmTask* __restrict__ tasks, int q) {
     __shared__ double2 As[16][33];
     __shared__ double2 Bs[32][17];
@@ -283,6 +340,43 @@ int upload(ls_handle* h, const std::vector<T>& v, T** dptr, size_t* cap) {
     }
     LS_CUDA(cudaMemcpyAsync(*dptr, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, h->stream));
     return LS_OK;
+}
+
+// All tasks of a launch.  Whole-width CTAs from 600 tasks on (about four CTAs per SM with
+// their row chunks), tiles below, where 9 of them per matrix spread a small level further.
+template <int RT>
+int gemm_wide(ls_handle* h, const GemmTask* tasks, unsigned nt, int q) {
+    const int rows = 256 / q * RT;
+    LS_LAUNCH(h, k_gemm_wide<RT>, dim3(nt, (unsigned)((q + rows - 1) / rows)), 256,
+              sizeof(double2) * 16 * (size_t)(rows + q), tasks, q);
+    return LS_OK;
+}
+int gemm_all(ls_handle* h, const GemmTask* tasks, size_t nt, int q) {
+    if (nt == 0) return LS_OK;
+    // rows per thread: the fewest padded rows over the chunks
+    const int CG = 256 / q, tiles = (q + 31) / 32;
+    int best = 8, pad = 1 << 30;
+    for (int rt = 6; rt <= 11; ++rt) {
+        const int rows = CG * rt, p = (q + rows - 1) / rows * rows;
+        if (p <= pad) {
+            pad = p;
+            best = rt;
+        }
+    }
+    // the form that keeps more lanes busy
+    const double wide = (double)q / pad * q * CG / 256.0, tiled = (double)q * q / (1024.0 * tiles * tiles);
+    if (nt < 600 || wide <= tiled) {
+        LS_LAUNCH(h, k_gemm, dim3((unsigned)nt, tiles * tiles), 256, 0, tasks, q);
+        return LS_OK;
+    }
+    switch (best) {
+        case 6: return gemm_wide<6>(h, tasks, (unsigned)nt, q);
+        case 7: return gemm_wide<7>(h, tasks, (unsigned)nt, q);
+        case 8: return gemm_wide<8>(h, tasks, (unsigned)nt, q);
+        case 9: return gemm_wide<9>(h, tasks, (unsigned)nt, q);
+        case 10: return gemm_wide<10>(h, tasks, (unsigned)nt, q);
+        default: return gemm_wide<11>(h, tasks, (unsigned)nt, q);
+    }
 }
 
 struct Scratch {
@@ -436,9 +530,8 @@ int factor_direction(ls_handle* h, int dir, Scratch& S) {
                 }
             }
         }
-        const int tiles = (q + 31) / 32;
         LS_TRY(upload(h, gt, &S.gem, &S.gem_cap));
-        if (!gt.empty()) LS_LAUNCH(h, k_gemm, dim3((unsigned)gt.size(), tiles * tiles), 256, 0, S.gem, q);
+        LS_TRY(gemm_all(h, S.gem, gt.size(), q));
         // 3) reduced blocks for level k+1 into work[nxt]
         std::vector<GemmTask> rt;
         rt.reserve((size_t)L * nnext * 3);
@@ -470,7 +563,7 @@ int factor_direction(ls_handle* h, int dir, Scratch& S) {
                 }
             }
         LS_TRY(upload(h, rt, &S.gem, &S.gem_cap));
-        if (!rt.empty()) LS_LAUNCH(h, k_gemm, dim3((unsigned)rt.size(), tiles * tiles), 256, 0, S.gem, q);
+        LS_TRY(gemm_all(h, S.gem, rt.size(), q));
         cur = nxt;
     }
     // top block: the single block of level K (level 0 if n == 1 is excluded by n >= 8)

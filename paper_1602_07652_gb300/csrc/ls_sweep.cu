@@ -239,6 +239,10 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     }
     pdl_wait();
 
+    // In the set-up's FP64 steps on the identity's columns most vectors are still zero on the
+    // forward way: their products are left out.
+    constexpr bool kSparse = sizeof(T) == 8 && NB == 8;
+    bool nonzero = false;
     // vectors, row r = tid % 128, members and slots alternating between the halves of the CTA
     if constexpr (MODE == 6) {
         for (int c = tid; c < ncol; c += kMvThreads) {
@@ -286,6 +290,7 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
                 }
             }
             vin[(size_t)p * q + r] = val;
+            if (kSparse) nonzero = nonzero || val.x != T(0) || val.y != T(0);
         }
         if ((MODE == 0 || MODE == 5) && sp == 0 && tid < nb) a.src.keep_trace(MODE == 0 ? j : 2 * j, b0 + tid);
     }
@@ -298,12 +303,14 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     };
     C base = czero<C>();
     if (tid < nout) base = base_of(NB == 1 ? 0 : tid / nr, r0 + (NB == 1 ? tid : tid % nr));
-    __syncthreads();
+    int cend = ncol;
+    if (kSparse) cend = __syncthreads_or(nonzero) ? ncol : 0;
+    else __syncthreads();
     if (!kEarly && !(sizeof(T) == 8 && gridDim.x <= 304)) pdl_trigger();   // else at its end
     C part[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) part[b] = czero<C>();
-    for (int c0 = cg; c0 < ncol; c0 += CG * PF) {
+    for (int c0 = cg; c0 < cend; c0 += CG * PF) {
 #pragma unroll
         for (int u = 0; u < PF; ++u) {
             const int c = c0 + u * CG;
