@@ -18,6 +18,7 @@
 // written.
 #pragma once
 
+#include "ls_f32x2.cuh"
 #include "ls_internal.cuh"
 
 struct __align__(8) dfl {
@@ -109,27 +110,94 @@ struct SrcIncDf {
     const cdfl* ez;
     int n;
     template <typename C>
-    __device__ __forceinline__ cdfl load(int z, int x) const {
-        return m[(size_t)z * n + x] * (ldg_c(&ex[x]) * ldg_c(&ez[z]));
+    __device__ __forceinline__ C load(int z, int x) const {
+        return ccast<C>(m[(size_t)z * n + x] * (ldg_c(&ex[x]) * ldg_c(&ez[z])));
     }
 };
 
-// d * exp(-DIR 2 pi i idx / 16) (the in-register DFT's constant rotations, found by argument-
-// dependent lookup): the odd multiples of pi/4 as one sum and one product per component (18
-// operations instead of 25), the others as one two-term product sum (20).
-__device__ __forceinline__ dfl df_cos16(int i) {   // cos(2 pi i / 16), i in [0, 8]
-    return i == 1 ? dfl(0.92387953251128675613) : i == 3 ? dfl(0.38268343236508977173)
-         : i == 5 ? dfl(-0.38268343236508977173) : i == 7 ? dfl(-0.92387953251128675613) : dfl(0.f, 0.f);
+// A double-float complex value with its components side by side, hi = (x.hi, y.hi) and lo =
+// (x.lo, y.lo), so that the error-free transformations above run on both at once in packed
+// FP32x2 instructions: 11 per complex sum, 19 per product (22 and 38 one component at a
+// time).  Same operations in the same order, except that a product's two terms enter each
+// component's error in the other order for the imaginary part.
+struct __align__(16) cdp {
+    F2 hi, lo;
+};
+template <> __host__ __device__ __forceinline__ cdp czero<cdp>() { return cdp{F2{0ull}, F2{0ull}}; }
+__device__ __forceinline__ cdp cdp_fast_two_sum(F2 a, F2 b) {   // |a| >= |b|
+    const F2 s = add2(a, b);
+    return cdp{s, sub2(b, sub2(s, a))};
 }
+__device__ __forceinline__ cdp cdp_two_sum(F2 a, F2 b) {
+    const F2 s = add2(a, b), bb = sub2(s, a);
+    return cdp{s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ cdp operator+(cdp a, cdp b) {
+    const cdp s = cdp_two_sum(a.hi, b.hi);
+    return cdp_fast_two_sum(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ cdp operator-(cdp a) { return cdp{neg2(a.hi), neg2(a.lo)}; }
+__device__ __forceinline__ cdp operator-(cdp a, cdp b) {
+    const F2 nb = neg2(b.hi);
+    const cdp s = cdp_two_sum(a.hi, nb);
+    return cdp_fast_two_sum(s.hi, add2(s.lo, sub2(a.lo, b.lo)));
+}
+__device__ __forceinline__ F2 f2swap(F2 a) {
+    float x, y;
+    f2split(a, x, y);
+    return f2(y, x);
+}
+// a w, w = c + i s: (x c, y c) + (-y s, x s)
+__device__ __forceinline__ cdp operator*(cdp a, cdfl w) {
+    const F2 ch = f2s(w.x.hi), cl = f2s(w.x.lo), sh = f2(-w.y.hi, w.y.hi), sl = f2(-w.y.lo, w.y.lo);
+    const F2 bh = f2swap(a.hi), bl = f2swap(a.lo);
+    const F2 p = mul2(a.hi, ch), q = mul2(bh, sh);
+    const cdp s = cdp_two_sum(p, q);
+    F2 e = add2(fma2(a.hi, ch, neg2(p)), fma2(bh, sh, neg2(q)));
+    e = fma2(a.hi, cl, e);
+    e = fma2(a.lo, ch, e);
+    e = fma2(bh, sl, e);
+    e = fma2(bl, sh, e);
+    return cdp_fast_two_sum(s.hi, add2(s.lo, e));
+}
+__device__ __forceinline__ cdp operator*(dfl r, cdp a) {
+    const F2 h = f2s(r.hi), p = mul2(a.hi, h);
+    F2 e = fma2(a.hi, h, neg2(p));
+    e = fma2(a.hi, f2s(r.lo), e);
+    e = fma2(a.lo, h, e);
+    return cdp_fast_two_sum(p, e);
+}
+// d * exp(-DIR 2 pi i idx / 16) for even idx < 8 (radix <= 8; found by argument-dependent
+// lookup): an odd multiple of pi/4 is one sum and one real product
 template <int DIR>
-__device__ __forceinline__ cdfl rot16(cdfl d, int idx) {
-    const dfl h(0.70710678118654752440);
+__device__ __forceinline__ cdp rot16(cdp d, int idx) {
     if (idx == 0) return d;
-    if (idx == 4) return DIR > 0 ? cdfl{d.y, -d.x} : cdfl{-d.y, d.x};
-    if (idx == 2) return DIR > 0 ? cdfl{(d.x + d.y) * h, (d.y - d.x) * h} : cdfl{(d.x - d.y) * h, (d.x + d.y) * h};
-    if (idx == 6) return DIR > 0 ? cdfl{(d.y - d.x) * h, -((d.x + d.y) * h)} : cdfl{-((d.x + d.y) * h), (d.x - d.y) * h};
-    const dfl c = df_cos16(idx), s = df_cos16(idx <= 4 ? 4 - idx : idx - 4);
-    if (DIR > 0) return cdfl{df_dot2(d.x, c, d.y, s), df_dot2(d.y, c, -d.x, s)};
-    return cdfl{df_dot2(d.x, c, -d.y, s), df_dot2(d.y, c, d.x, s)};
+    const auto quarter = [](cdp a) {   // a * (-+ i)
+        float xh, yh, xl, yl;
+        f2split(a.hi, xh, yh);
+        f2split(a.lo, xl, yl);
+        return DIR > 0 ? cdp{f2(yh, -xh), f2(yl, -xl)} : cdp{f2(-yh, xh), f2(-yl, xl)};
+    };
+    if (idx == 4) return quarter(d);
+    const cdp t = dfl(0.70710678118654752440) * (d + quarter(d));
+    return idx == 2 ? t : quarter(t);
+}
+template <> __host__ __device__ __forceinline__ cdp ccast<cdp, cdfl>(cdfl a) {
+#ifdef __CUDA_ARCH__
+    return cdp{f2(a.x.hi, a.y.hi), f2(a.x.lo, a.y.lo)};
+#else
+    return cdp{};
+#endif
+}
+template <> __host__ __device__ __forceinline__ cdp ccast<cdp, double2>(double2 a) { return ccast<cdp>(ccast<cdfl>(a)); }
+template <> __host__ __device__ __forceinline__ double2 ccast<double2, cdp>(cdp a) {
+#ifdef __CUDA_ARCH__
+    float xh, yh, xl, yl;
+    f2split(a.hi, xh, yh);
+    f2split(a.lo, xl, yl);
+    return make_double2(dbl_of(dfl(xh, xl)), dbl_of(dfl(yh, yl)));
+#else
+    return make_double2(0.0, 0.0);
+#endif
 }
 #endif

@@ -383,6 +383,27 @@ __global__ void k_twiddles(int P, double2* tw64, float2* tw32) {
     tw32[m] = make_float2((float)c, (float)-s);
 }
 
+// the twiddles of the passes specialised on P, stage by stage (wide_tw_off): gathered from the
+// table tw[m] = exp(-2 pi i m / P) into out[0 .. P) (forward) and out[P .. 2 P) (inverse)
+template <typename W>
+__global__ void k_wide_twiddles(int lp, const W* __restrict__ tw, W* __restrict__ out) {
+    const int P = 1 << lp, ns = (lp + 2) / 3, lrl = lp - 3 * (ns - 1);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 2 * P) return;
+    const bool inverse = i >= P;
+    int o = inverse ? i - P : i;
+    for (int S = 1; S < ns; ++S) {
+        const int ls = inverse ? lrl + 3 * (S - 1) : 3 * S, lr = inverse || S < ns - 1 ? 3 : lrl;
+        const int cnt = ((1 << lr) - 1) << ls;
+        if (o < cnt) {
+            const int r = (o >> ls) + 1, k = o & ((1 << ls) - 1);
+            out[i] = tw[(k * r) << (lp - ls - lr)];
+            return;
+        }
+        o -= cnt;
+    }
+}
+
 __global__ void k_incident_factors(int n, double wh, double cth, double sth, double2* ex, double2* ez) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -488,6 +509,10 @@ int ls_fft_init(ls_handle* h) {
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<float2>>, row_smem32(P)));
     LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<double2>>, row_smem32(P)));
     if (h->lp >= 6) {
+        LS_CUDA(cudaMalloc(&h->tww64, sizeof(double2) * 2 * P));
+        LS_CUDA(cudaMalloc(&h->twwdf, sizeof(cdfl) * 2 * P));
+        LS_LAUNCH(h, k_wide_twiddles<double2>, (2 * P + 255) / 256, 256, 0, h->lp, h->tw64, h->tww64);
+        LS_LAUNCH(h, k_wide_twiddles<cdfl>, (2 * P + 255) / 256, 256, 0, h->lp, h->twdf, h->twwdf);
         LS_TRY(ls_wide64_init());
         LS_TRY(ls_widedf_init());
     }

@@ -39,6 +39,7 @@
 
 #include <mutex>
 
+#include "ls_f32x2.cuh"
 #include "ls_fft_common.cuh"
 
 namespace {
@@ -133,49 +134,8 @@ __device__ __forceinline__ void stage(V (&v)[CW][E], int j, const float2* __rest
 
 // ------------------------------------------------- two columns per FP32x2 instruction
 // The column pass applies identical operations to the two columns of a tile, so a
-// pair of values (column 0, column 1) can travel in one 64-bit register and be
-// added, multiplied and fused-multiply-added by the packed FP32 instructions of
-// sm_100+ (add/sub/mul/fma .rn.f32x2: two IEEE single-precision operations, each
-// rounded to nearest, in one instruction).  CP holds a complex value of both
-// columns: x = (re0, re1), y = (im0, im1).
-struct F2 {
-    unsigned long long r;
-};
-__device__ __forceinline__ F2 f2(float lo, float hi) {
-    F2 o;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(o.r) : "f"(lo), "f"(hi));
-    return o;
-}
-__device__ __forceinline__ F2 f2s(float a) { return f2(a, a); }
-__device__ __forceinline__ void f2split(F2 a, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.r));
-}
-__device__ __forceinline__ F2 add2(F2 a, F2 b) {
-    F2 o;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(o.r) : "l"(a.r), "l"(b.r));
-    return o;
-}
-__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
-    F2 o;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(o.r) : "l"(a.r), "l"(b.r));
-    return o;
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-    F2 o;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(o.r) : "l"(a.r), "l"(b.r));
-    return o;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {  // a b + c
-    F2 o;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(o.r) : "l"(a.r), "l"(b.r), "l"(c.r));
-    return o;
-}
-__device__ __forceinline__ F2 neg2(F2 a) {  // flips both sign bits
-    F2 o;
-    asm("xor.b64 %0, %1, 0x8000000080000000;" : "=l"(o.r) : "l"(a.r));
-    return o;
-}
-
+// pair of values (column 0, column 1) can travel in one 64-bit register (ls_f32x2.cuh).
+// CP holds a complex value of both columns: x = (re0, re1), y = (im0, im1).
 struct CP {
     F2 x, y;
 };
@@ -389,7 +349,7 @@ __global__ void __launch_bounds__(Geo<LP, LE>::THREADS, MINB) k_cols16(int nin, 
     inv_stages<LP, LE, 0, false>(v, buf, j, tw);
     pdl_trigger();
 #pragma unroll
-    for (int t = 0; t < E; ++t) {
+    for (int t = 0; t < E / 2; ++t) {   // nout <= P / 2: the other outputs are never formed
         const int z = j + t * T;
         if (z < nout) *reinterpret_cast<EL*>(X + (size_t)z * P + kx0) = Elem<CW>::pack(v, t);
     }
@@ -535,7 +495,7 @@ __global__ void __launch_bounds__(Geo<LP, LE, kTmaCta>::THREADS, MINB) k_cols16_
     pdl_trigger();
     __syncthreads();  // every thread is done with the exchange buffer
 #pragma unroll
-    for (int t = 0; t < E; ++t) {
+    for (int t = 0; t < E / 2; ++t) {   // nbox * BR <= P / 2: the other outputs are never formed
         const int z = j + t * T;
         if (z < nbox * BR) buf[z] = Elem<CW>::pack(v, t);
     }
@@ -639,7 +599,7 @@ __global__ void __launch_bounds__(Geo<LP, LE, kTmaCta>::THREADS, MINB) k_cols16_
     pdl_trigger();
     __syncthreads();
 #pragma unroll
-    for (int t = 0; t < E; ++t) {
+    for (int t = 0; t < E / 2; ++t) {   // nbox * BR <= P / 2: the other outputs are never formed
         const int z = j + t * T;
         if (z < nbox * BR) stg[z] = f4_of(v[0][t]);
     }

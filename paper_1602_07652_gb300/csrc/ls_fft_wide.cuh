@@ -30,22 +30,32 @@ struct GeoW {
     static constexpr int THREADS = T >= 128 ? T : 128, G = THREADS / T;
     static constexpr int NS = (LP + 2) / 3, LRL = LP - 3 * (NS - 1);   // stages, log2 of the last radix
     static constexpr int SLOTS = P + P / 8;                // a padding slot every 8 elements
-    static constexpr int MINB = 1024 / THREADS;
+    static constexpr int MINB = (LRL == 1 ? 768 : 1024) / THREADS;   // (a last radix of 2 needs 80 registers)
     static constexpr size_t smem = (size_t)G * SLOTS * 16;
 };
 __device__ __forceinline__ int pad8(int i) { return i + (i >> 3); }
 
-// v[e R + r] *= exp(-DIR 2 pi i k r / 2^(LS+LR)); tw[m] = exp(-2 pi i m / P)
-template <int LR, int LS, int DIR, int LP, bool HZ, typename C>
-__device__ __forceinline__ void stage_w(C (&v)[8], int j, const C* __restrict__ tw) {
-    constexpr int R = 1 << LR, SH = LP - LS - LR, T = GeoW<LP>::T;
+// Twiddles stage by stage, exp(-2 pi i k r / 2^(LS+LR)) at [offset of the stage][r - 1][k], the
+// forward stages in the first P entries and the inverse ones in the next P: a warp's factors
+// are consecutive.  In the one table exp(-2 pi i m / P) they lie up to a line apart, and a
+// load took up to 32 wavefronts of the LSU (half of the double-float column pass's).
+constexpr int wide_tw_off(bool inverse, int lrl, int S) {   // offset of stage S >= 1
+    int o = 0;
+    for (int s = 1; s < S; ++s) o += 7 << (inverse ? lrl + 3 * (s - 1) : 3 * s);
+    return o;
+}
+
+// One stage: v[e R + r] *= exp(-DIR 2 pi i k r / 2^(LS+LR)), then the DFTs; tw: the stage's factors
+template <int LR, int LS, int DIR, int LP, bool HZ, typename C, typename W>
+__device__ __forceinline__ void stage_w(C (&v)[8], int j, const W* __restrict__ tw) {
+    constexpr int R = 1 << LR, T = GeoW<LP>::T;
 #pragma unroll
     for (int e = 0; e < 8 / R; ++e) {
         if constexpr (LS > 0) {
             const int k = (j + e * T) & ((1 << LS) - 1);
 #pragma unroll
             for (int r = 1; r < R; ++r) {
-                C w = ldg_c(&tw[(k * r) << SH]);
+                W w = ldg_c(&tw[((r - 1) << LS) + k]);
                 if (DIR < 0) w.y = -w.y;
                 v[e * R + r] = v[e * R + r] * w;
             }
@@ -74,30 +84,30 @@ __device__ __forceinline__ void exchange_w(C (&v)[8], C* buf, int j) {
 }
 
 // Forward: in v[t] = x[j + t T] (t < 4; the rest is zero), out v[e R + r] = X[j + e T + r P/R], R = 2^LRL
-template <int LP, int S, bool FIRST, typename C>
-__device__ __forceinline__ void fwd_w(C (&v)[8], C* buf, int j, const C* __restrict__ tw) {
+template <int LP, int S, bool FIRST, typename C, typename W>
+__device__ __forceinline__ void fwd_w(C (&v)[8], C* buf, int j, const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int LR = S < Gm::NS - 1 ? 3 : Gm::LRL;
     if constexpr (S > 0) exchange_w<3, 3 * (S - 1), LR, LP, FIRST && S == 1>(v, buf, j);
-    stage_w<LR, 3 * S, +1, LP, S == 0>(v, j, tw);
+    stage_w<LR, 3 * S, +1, LP, S == 0>(v, j, tw + wide_tw_off(false, Gm::LRL, S));
     if constexpr (S + 1 < Gm::NS) fwd_w<LP, S + 1, FIRST>(v, buf, j, tw);
 }
 // Inverse (unnormalised): the layout fwd_w leaves -> v[t] = x[j + t T]
-template <int LP, int S, bool FIRST, typename C>
-__device__ __forceinline__ void inv_w(C (&v)[8], C* buf, int j, const C* __restrict__ tw) {
+template <int LP, int S, bool FIRST, typename C, typename W>
+__device__ __forceinline__ void inv_w(C (&v)[8], C* buf, int j, const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int LR = S == 0 ? Gm::LRL : 3, LS = S == 0 ? 0 : Gm::LRL + 3 * (S - 1);
     if constexpr (S > 0) {
         constexpr int LRP = S == 1 ? Gm::LRL : 3, LSP = S == 1 ? 0 : Gm::LRL + 3 * (S - 2);
         exchange_w<LRP, LSP, LR, LP, FIRST && S == 1>(v, buf, j);
     }
-    stage_w<LR, LS, -1, LP, false>(v, j, tw);
+    stage_w<LR, LS, -1, LP, false>(v, j, tw + Gm::P + wide_tw_off(true, Gm::LRL, S));
     if constexpr (S + 1 < Gm::NS) inv_w<LP, S + 1, FIRST>(v, buf, j, tw);
 }
 
-template <int LP, typename C, class Src>
+template <int LP, typename C, typename W, class Src>
 __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows_fwd(int n, Src src, C* __restrict__ X,
-                                                                                 const C* __restrict__ tw) {
+                                                                                 const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int T = Gm::T, R = 1 << Gm::LRL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -121,10 +131,10 @@ __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows
         for (int r = 0; r < R; ++r) o[j + e * T + r * (Gm::P / R)] = v[e * R + r];
 }
 
-template <int LP, typename C>
+template <int LP, typename C, typename W>
 __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_cols(int n, C* __restrict__ X,
-                                                                             const C* __restrict__ ghat,
-                                                                             const C* __restrict__ tw) {
+                                                                             const W* __restrict__ ghat,
+                                                                             const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int P = Gm::P, T = Gm::T, R = 1 << Gm::LRL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -134,7 +144,7 @@ __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_cols
     const int lin = blockIdx.x * Gm::G + grp;
     const int kx = (lin & 1) ? (P - 1 - (lin >> 1)) : (lin >> 1);
     C* col = X + kx;
-    const C* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * (P / 2 + 1);
+    const W* g = ghat + (size_t)(kx <= P / 2 ? kx : P - kx) * (P / 2 + 1);
     pdl_wait();
     C v[8];
 #pragma unroll
@@ -159,9 +169,9 @@ __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_cols
     }
 }
 
-template <int LP, typename C, class Dst>
+template <int LP, typename C, typename W, class Dst>
 __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows_inv(int n, const C* __restrict__ X, Dst dst,
-                                                                                 const C* __restrict__ tw) {
+                                                                                 const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int T = Gm::T, R = 1 << Gm::LRL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -185,39 +195,39 @@ __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows
     }
 }
 
-template <int LP, typename C, class Src, class Dst>
-int wide_lp(ls_handle* h, const Src& src, const Dst& dst, const C* ghat, const C* tw) {
+template <int LP, typename C, typename W, class Src, class Dst>
+int wide_lp(ls_handle* h, const Src& src, const Dst& dst, const W* ghat, const W* tw) {
     using Gm = GeoW<LP>;
     const int n = h->n;
     C* X = static_cast<C*>(h->fftws);
     const dim3 rows((unsigned)((n + Gm::G - 1) / Gm::G)), threads(Gm::THREADS);
-    LS_TRY(ls_launch_pdl(h, k_wide_rows_fwd<LP, C, Src>, rows, threads, Gm::smem, n, src, X, tw));
-    LS_TRY(ls_launch_pdl(h, k_wide_cols<LP, C>, dim3(Gm::P / Gm::G), threads, Gm::smem, n, X, ghat, tw));
-    return ls_launch_pdl(h, k_wide_rows_inv<LP, C, Dst>, rows, threads, Gm::smem, n, static_cast<const C*>(X), dst, tw);
+    LS_TRY(ls_launch_pdl(h, k_wide_rows_fwd<LP, C, W, Src>, rows, threads, Gm::smem, n, src, X, tw));
+    LS_TRY(ls_launch_pdl(h, k_wide_cols<LP, C, W>, dim3(Gm::P / Gm::G), threads, Gm::smem, n, X, ghat, tw));
+    return ls_launch_pdl(h, k_wide_rows_inv<LP, C, W, Dst>, rows, threads, Gm::smem, n, static_cast<const C*>(X), dst, tw);
 }
 
-template <typename C, class Src, class Dst>
-int wide_apply(ls_handle* h, const Src& src, const Dst& dst, const C* ghat, const C* tw) {
+template <typename C, typename W, class Src, class Dst>
+int wide_apply(ls_handle* h, const Src& src, const Dst& dst, const W* ghat, const W* tw) {
     switch (h->lp) {
-        case 6: return wide_lp<6>(h, src, dst, ghat, tw);
-        case 7: return wide_lp<7>(h, src, dst, ghat, tw);
-        case 8: return wide_lp<8>(h, src, dst, ghat, tw);
-        case 9: return wide_lp<9>(h, src, dst, ghat, tw);
-        case 10: return wide_lp<10>(h, src, dst, ghat, tw);
-        case 11: return wide_lp<11>(h, src, dst, ghat, tw);
-        case 12: return wide_lp<12>(h, src, dst, ghat, tw);
+        case 6: return wide_lp<6, C>(h, src, dst, ghat, tw);
+        case 7: return wide_lp<7, C>(h, src, dst, ghat, tw);
+        case 8: return wide_lp<8, C>(h, src, dst, ghat, tw);
+        case 9: return wide_lp<9, C>(h, src, dst, ghat, tw);
+        case 10: return wide_lp<10, C>(h, src, dst, ghat, tw);
+        case 11: return wide_lp<11, C>(h, src, dst, ghat, tw);
+        case 12: return wide_lp<12, C>(h, src, dst, ghat, tw);
         default: return LS_EINVAL;
     }
 }
 
 // dynamic shared memory above 48 KB (P = 4096 only)
-template <typename C, class Src, class Dst>
+template <typename C, typename W, class Src, class Dst>
 int wide_optin() {
     using Gm = GeoW<12>;
     static_assert(GeoW<11>::smem <= 48 * 1024, "only P = 4096 needs the opt-in");
-    LS_CUDA(cudaFuncSetAttribute(k_wide_rows_fwd<12, C, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
-    LS_CUDA(cudaFuncSetAttribute(k_wide_cols<12, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
-    LS_CUDA(cudaFuncSetAttribute(k_wide_rows_inv<12, C, Dst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
+    LS_CUDA(cudaFuncSetAttribute(k_wide_rows_fwd<12, C, W, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
+    LS_CUDA(cudaFuncSetAttribute(k_wide_cols<12, C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
+    LS_CUDA(cudaFuncSetAttribute(k_wide_rows_inv<12, C, W, Dst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::smem));
     return LS_OK;
 }
 

@@ -3,12 +3,12 @@
 #include "ls_fft_wide.cuh"
 
 int ls_widedf_init() {
-    LS_TRY((wide_optin<cdfl, SrcMU<dfl, double2>, DstApply<double2>>()));
-    return wide_optin<cdfl, SrcIncDf, DstRhs>();
+    LS_TRY((wide_optin<cdp, cdfl, SrcMU<dfl, double2>, DstApply<double2>>()));
+    return wide_optin<cdp, cdfl, SrcIncDf, DstRhs>();
 }
 int ls_widedf_apply(ls_handle* h, const double2* u, double2* y) {
-    return wide_apply<cdfl>(h, SrcMU<dfl, double2>{h->mdf, u, h->n}, DstApply<double2>{u, y, h->n}, h->ghatdf, h->twdf);
+    return wide_apply<cdp>(h, SrcMU<dfl, double2>{h->mdf, u, h->n}, DstApply<double2>{u, y, h->n}, h->ghatdf, h->twwdf);
 }
 int ls_widedf_rhs(ls_handle* h, double2* f) {
-    return wide_apply<cdfl>(h, SrcIncDf{h->mdf, h->incxdf, h->inczdf, h->n}, DstRhs{f, h->n}, h->ghatdf, h->twdf);
+    return wide_apply<cdp>(h, SrcIncDf{h->mdf, h->incxdf, h->inczdf, h->n}, DstRhs{f, h->n}, h->ghatdf, h->twwdf);
 }

@@ -220,6 +220,8 @@ struct ls_handle {
     struct dfl* mdf = nullptr;
     struct cdfl* ghatdf = nullptr;
     struct cdfl* twdf = nullptr;
+    double2* tww64 = nullptr;      // twiddles of the passes specialised on P (ls_fft_wide.cuh)
+    struct cdfl* twwdf = nullptr;
     struct cdfl* incxdf = nullptr;
     struct cdfl* inczdf = nullptr;
     int dfloat = 0;            // 1 (LS_MIXED default): refinement residuals and incident
