@@ -33,7 +33,8 @@
 // start instead crowds the SMs that are idle then (512^2: 24 us against 15).  With this, the
 // kernels for 32 <= P < 256 and the default tile shapes (ls_fft16_default), back-to-back calls
 // went from 20.5 to 6.3 us (64^2), 21.6 to 8.9 (256^2), 24.6 to 14.9 (512^2), 57.7 to 41.6
-// (1024^2) and 199 to 141 us (2048^2).
+// (1024^2) and 199 to 141 us (2048^2); with the stage-by-stage twiddles and only the outputs
+// that are stored to 8.3 (256^2), 14.0, 37.3 and 123.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -87,21 +88,49 @@ __device__ __forceinline__ float2 ld_tw(const float2* __restrict__ tw, int m) {
     return w;
 }
 
+// The twiddles that the stages load (k < 2^LS, r = 1, 2, 4, 8) lie stage by stage: factor
+// exp(-2 pi i k 2^b / 2^(LS+LR)) at [stage][b][k], so that a warp's factors are consecutive; in
+// the one table exp(-2 pi i m / P) they are up to a line apart and a load took 16 to 32
+// wavefronts of the LSU, which the exchanges need.  Four tables of P entries: radix 16
+// forward, inverse, radix 8 forward, inverse (k_fft16_twiddles).
+constexpr int tw16_off(int lp, int le, int dir, int ls) {   // offset of the stage at 2^ls
+    const int lrl = lp - le * ((lp + le - 1) / le - 1);
+    int o = ((le == 4 ? 0 : 2) + (dir < 0 ? 1 : 0)) << lp;
+    for (int l = dir > 0 ? le : lrl; l < ls; l += le) o += le << l;
+    return o;
+}
+__global__ void k_fft16_twiddles(int lp, const float2* __restrict__ tw, float2* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 4 << lp) return;
+    const int t = i >> lp, le = t < 2 ? 4 : 3, ns = (lp + le - 1) / le, lrl = lp - le * (ns - 1);
+    int o = i & ((1 << lp) - 1);
+    for (int S = 1; S < ns; ++S) {
+        const int ls = (t & 1) ? lrl + le * (S - 1) : le * S, lr = (t & 1) || S < ns - 1 ? le : lrl;
+        if (o < lr << ls) {
+            const int b = o >> ls, k = o & ((1 << ls) - 1);
+            out[i] = tw[(k << b) << (lp - ls - lr)];
+            return;
+        }
+        o -= lr << ls;
+    }
+}
+
 // v[c][e R + r] *= W^(k r), W = exp(-DIR 2 pi i / 2^(LS+LR)), r = 1..R-1.
-// tw[m] = exp(-2 pi i m / P), so W^s = tw[s << (LP - LS - LR)].
+// tw: the tables above, or for P < 256 tw[m] = exp(-2 pi i m / P).
 template <int LR, int LS, int DIR, int LP, int CW, int E, typename V>
 __device__ __forceinline__ void twiddle(V (&v)[CW][E], int e, int k, const float2* __restrict__ tw) {
     constexpr int R = 1 << LR;
     constexpr int SH = LP - LS - LR;
     float2 w[16];
-    w[1] = ld_tw<DIR>(tw, k << SH);
     if constexpr (LP < 8) {   // short transforms wait on latency, not on load slots: all from the table
 #pragma unroll
-        for (int r = 2; r < R; ++r) w[r] = ld_tw<DIR>(tw, (r * k) << SH);
+        for (int r = 1; r < R; ++r) w[r] = ld_tw<DIR>(tw, (r * k) << SH);
     } else {
-        if (R > 2) w[2] = ld_tw<DIR>(tw, (2 * k) << SH);
-        if (R > 4) w[4] = ld_tw<DIR>(tw, (4 * k) << SH);
-        if (R > 8) w[8] = ld_tw<DIR>(tw, (8 * k) << SH);
+        constexpr int O = tw16_off(LP, E == 16 ? 4 : 3, DIR, LS);
+        w[1] = ld_tw<DIR>(tw, O + k);
+        if (R > 2) w[2] = ld_tw<DIR>(tw, O + (1 << LS) + k);
+        if (R > 4) w[4] = ld_tw<DIR>(tw, O + (2 << LS) + k);
+        if (R > 8) w[8] = ld_tw<DIR>(tw, O + (3 << LS) + k);
         if (R > 2) w[3] = w[2] * w[1];
         if (R > 4) {
             w[5] = w[4] * w[1];
@@ -734,7 +763,7 @@ template <int LP, typename UIO>
 int apply_lp(ls_handle* h, const UIO* u, UIO* y, float2* X, int shape) {
     using Gm = Geo<LP, 4>;
     const int n = h->n;
-    const float2* tw = static_cast<const float2*>(h->tw32);
+    const float2* tw = LP < 8 ? h->tw32 : h->tww32;
     const float2* gh = static_cast<const float2*>(h->ghat32);
     const unsigned rows_grid = (unsigned)((n + Gm::G - 1) / Gm::G);
     SrcMU<float, UIO> src{h->m32, u, n};
@@ -805,6 +834,10 @@ bool ls_fft16_supported(const ls_handle* h, int shape) {
 int ls_fft16_default(const ls_handle* h) { return h->lp <= 9 ? 4 : 8; }
 
 int ls_fft16_init(ls_handle* h) {
+    if (h->lp >= 8 && h->lp <= 12) {
+        LS_CUDA(cudaMalloc(&h->tww32, sizeof(float2) * 4 * h->P));
+        LS_LAUNCH(h, k_fft16_twiddles, (unsigned)((4 * h->P + 255) / 256), 256, 0, h->lp, h->tw32, h->tww32);
+    }
     LS_TRY(optin_lp<8>());
     LS_TRY(optin_lp<9>());
     LS_TRY(optin_lp<10>());

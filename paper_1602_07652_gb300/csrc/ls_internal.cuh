@@ -215,6 +215,7 @@ struct ls_handle {
     float2* ghat32 = nullptr;
     double2* tw64 = nullptr;   // twiddles exp(-2 pi i m / P), m < P
     float2* tw32 = nullptr;
+    float2* tww32 = nullptr;   // the same stage by stage (ls_fft16.cu), 4 P entries
     // double-float copies (ls_dfloat.cuh) of the medium, the spectral quadrant, the
     // twiddles and the incident-wave factors: the FP64-accurate convolutions on the FP32 pipes
     struct dfl* mdf = nullptr;
