@@ -385,8 +385,8 @@ int ls_transpose64(ls_handle* h, const double2* a, double2* b);
 int ls_transpose64_b(ls_handle* h, const double2* a, double2* b, int nb);
 int ls_stencil_apply64(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y);
 int ls_stencil_apply_b(ls_handle* h, int dir, int withm, const double2* v, const double2* g, double2* y, int nb);
-int ls_stencil_refine_f32(ls_handle* h, int dir, const float2* v, const float2* g, float2* y, int nb);
-int ls_stencil_apply_f32(ls_handle* h, int dir, int mode, const float2* v, float2* y);
+int ls_stencil_refine_f32(ls_handle* h, const float2* v, const float2* g, float2* y, int nb);
+int ls_stencil_apply_f32(ls_handle* h, int mode, const float2* v, float2* y);
 // Krylov vectors in FP64 (double2) or FP32 (float2); dot products summed in FP64
 // One fused pass of a Gram-Schmidt step against nvec directions (ls_stencil.cu) for
 // members members[0..cnt) of a lockstep batch in one launch (member m: V and w at

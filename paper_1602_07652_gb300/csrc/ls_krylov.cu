@@ -92,7 +92,7 @@ int apply_op(ls_handle* h, Op op, const float2* x, float2* y) {
     }
     if (op == OP_C) {
         LS_TRY(ls_timing_begin(h));
-        LS_TRY(ls_stencil_apply_f32(h, 0, 1, x, y));
+        LS_TRY(ls_stencil_apply_f32(h, 1, x, y));
         return ls_timing_end(h, 3);
     }
     return LS_EINVAL;   // the FP64 apply takes FP64 vectors
@@ -164,7 +164,7 @@ int gs_chunk(ls_handle* h, const float2* v, float2* z, int cnt) {
     return LS_OK;
 }
 int stencil_A(ls_handle* h, const double2* v, double2* y) { return ls_stencil_apply(h, 0, 0, v, nullptr, y); }
-int stencil_A(ls_handle* h, const float2* v, float2* y) { return ls_stencil_apply_f32(h, 0, 0, v, y); }
+int stencil_A(ls_handle* h, const float2* v, float2* y) { return ls_stencil_apply_f32(h, 0, v, y); }
 
 template <typename VT>
 int apply_pc_b(ls_handle* h, Pc pc, VT* v, VT* z, int nb, const unsigned char* on, ls_stats* st) {

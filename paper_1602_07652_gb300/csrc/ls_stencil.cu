@@ -23,11 +23,14 @@ namespace {
 // arithmetic type) by loads that are all issued before the first store, so every
 // value of v and m is read from HBM about once.
 constexpr int kStX = 32, kStZ = 32, kStRows = 4;   // tile, rows per thread (threads 32 x 8)
-// VF, YF: element types of v and y (double2; float2 for the mixed Algorithm 2's fields,
-// which hold FP32 values: v is the FP32 sweep's result, y feeds the FP32 sweep).
-template <int MODE, typename R, typename VF = double2, typename YF = double2, typename GF = double2>  // 0: y = A v  1: y = C v  2: y = g - C v
+// VF, YF, GF, MT: element types of v, y, g and m (double2 and double; float2 and float for the
+// mixed solve's fields, which hold FP32 values: v is the FP32 sweep's result, y feeds the
+// FP32 sweep).  With FP32 fields nothing is widened: through FP64 and back (on the integer
+// pipes) and with the FP64 medium a 2048^2 apply took 54 us for 100 MB.
+template <int MODE, typename R, typename VF = double2, typename YF = double2, typename GF = double2,
+          typename MT = double>  // 0: y = A v  1: y = C v  2: y = g - C v
 __global__ void __launch_bounds__(256) k_stencil(int n, const StencilTables* __restrict__ tab,
-                                                 const double* __restrict__ m, const VF* __restrict__ v,
+                                                 const MT* __restrict__ m, const VF* __restrict__ v,
                                                  const GF* __restrict__ g, YF* __restrict__ y) {
     using CR = cpx_t<R>;
     constexpr int HX = kStX + 2, HZ = kStZ + 2, HN = HX * HZ;
@@ -49,13 +52,13 @@ __global__ void __launch_bounds__(256) k_stencil(int n, const StencilTables* __r
     constexpr int PER = (HN + 255) / 256;   // halo tile elements per thread
     const VF vz = {};
     VF vv[PER];
-    double mv[PER];
+    MT mv[PER];
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         const int e = tid + u * 256, hz = e / HX, hx = e % HX, x = x0 + hx, z = z0 + hz;
         const bool in = e < HN && x >= 0 && x < n && z >= 0 && z < n;
         vv[u] = in ? __ldg(&v[(size_t)z * n + x]) : vz;
-        if (MODE >= 1) mv[u] = in ? __ldg(&m[(size_t)z * n + x]) : 0.0;
+        if (MODE >= 1) mv[u] = in ? __ldg(&m[(size_t)z * n + x]) : MT(0);
     }
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
@@ -63,7 +66,7 @@ __global__ void __launch_bounds__(256) k_stencil(int n, const StencilTables* __r
         if (e < HN) {
             sv[e / HX][e % HX] = ccast<CR>(vv[u]);
             if constexpr (MODE >= 1) {
-                if constexpr (sizeof(R) == 4) sm[e / HX][e % HX] = d2f_rn(mv[u]);
+                if constexpr (sizeof(R) == 4 && sizeof(MT) == 8) sm[e / HX][e % HX] = d2f_rn(mv[u]);
                 else sm[e / HX][e % HX] = mv[u];
             }
         }
@@ -96,9 +99,13 @@ __global__ void __launch_bounds__(256) k_stencil(int n, const StencilTables* __r
             }
         }
         const size_t k = (size_t)j * n + i;
-        double2 out = ccast<double2>(acc);
-        if (MODE == 2) out = ccast<double2>(__ldg(&g[k])) - out;
-        y[k] = ccast<YF>(out);
+        if constexpr (sizeof(YF) == 8 && sizeof(GF) == 8 && sizeof(R) == 4) {   // FP32 throughout
+            y[k] = MODE == 2 ? __ldg(&g[k]) - acc : acc;
+        } else {
+            double2 out = ccast<double2>(acc);
+            if (MODE == 2) out = ccast<double2>(__ldg(&g[k])) - out;
+            y[k] = ccast<YF>(out);
+        }
     }
 }
 
@@ -403,26 +410,25 @@ int ls_stencil_apply_b(ls_handle* h, int dir, int mode, const double2* v, const 
 
 // Algorithm 2's refinement residual e = g - C u1 in mixed precision, u1 and e in FP32
 // storage (their values are FP32 either way); FP32 coefficients and sums.
-int ls_stencil_refine_f32(ls_handle* h, int dir, const float2* v, const float2* g, float2* y, int nb) {
+int ls_stencil_refine_f32(ls_handle* h, const float2* v, const float2* g, float2* y, int nb) {
     const int n = h->n;
     const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), nb);
     const dim3 block(kStX, 256 / kStX);
-    const double* m = dir == 0 ? h->m64 : h->mT64;
-    LS_LAUNCH(h, (k_stencil<2, float, float2, float2, float2>), grid, block, 0, n, h->dtabs + dir, m, v, g, y);
+    LS_LAUNCH(h, (k_stencil<2, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, g, y);
     return LS_OK;
 }
 
 // y = A v (mode 0) or C v (mode 1) with FP32 vectors and FP32 arithmetic (the mixed
 // precision inner solve's operator)
-int ls_stencil_apply_f32(ls_handle* h, int dir, int mode, const float2* v, float2* y) {
+int ls_stencil_apply_f32(ls_handle* h, int mode, const float2* v, float2* y) {
     const int n = h->n;
     const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), 1);
     const dim3 block(kStX, 256 / kStX);
-    const double* m = dir == 0 ? h->m64 : h->mT64;
-    const StencilTables* tab = h->dtabs + dir;
-    const double2* none = nullptr;
-    if (mode == 0) LS_LAUNCH(h, (k_stencil<0, float, float2, float2>), grid, block, 0, n, tab, m, v, none, y);
-    else LS_LAUNCH(h, (k_stencil<1, float, float2, float2>), grid, block, 0, n, tab, m, v, none, y);
+    const float2* none = nullptr;
+    if (mode == 0)
+        LS_LAUNCH(h, (k_stencil<0, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, none, y);
+    else
+        LS_LAUNCH(h, (k_stencil<1, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, none, y);
     return LS_OK;
 }
 

@@ -518,16 +518,16 @@ __global__ void __launch_bounds__(256) k_gather(StripGeom g, const cpx_t<T>* __r
 }
 
 // The same tiles for all layers of a sweep at once, without the injections (the reduction
-// steps on the CUDA cores add them where level 0 reads the right-hand side): blockIdx.z =
-// member * L + layer.
+// steps on the CUDA cores add them where level 0 reads the right-hand side): blockIdx.x =
+// (member * L + layer) * column tiles + tile.
 template <typename T, bool TR, typename GF = double2>
 __global__ void __launch_bounds__(256) k_gather_all(StripGeom g, int L, const GF* __restrict__ gf,
                                                     cpx_t<T>* __restrict__ rhs, size_t SB) {
     using C = cpx_t<T>;
     __shared__ C tile[kGatherTile][kGatherTile + 1];   // [r - r0][i - i0]
     const int q = g.q, n = g.n, E = g.E, t = g.t;
-    const int b = blockIdx.z / L, l = blockIdx.z - b * L;
-    const int i0 = blockIdx.x * kGatherTile, r0 = blockIdx.y * kGatherTile;
+    const int it = (n + kGatherTile - 1) / kGatherTile, bl = blockIdx.x / it, b = bl / L, l = bl - b * L;
+    const int i0 = (blockIdx.x - bl * it) * kGatherTile, r0 = blockIdx.y * kGatherTile;
     gf += (size_t)b * n * n;
     rhs += (size_t)b * SB + (size_t)l * n * q;
     const int tx = threadIdx.x, ty = threadIdx.y;
@@ -586,33 +586,47 @@ __global__ void k_inject_up(StripGeom g, const cpx_t<T>* __restrict__ inj, int l
     sol[e] = val;
 }
 
-// v = rows 1..n of every layer's solution (concatenation); batch member b = blockIdx.y
+// v = rows 1..n of every layer's solution (concatenation); blocks as in k_gather_all, whose tiled
+// transpose this is the other way round: reads along r, writes along x.
 template <typename T, typename OF = double2>
-__global__ void k_scatter(StripGeom g, const cpx_t<T>* __restrict__ sol, size_t strip_stride, size_t SB,
-                          OF* __restrict__ v) {
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = g.n;
-    if (e >= (size_t)n * n) return;
-    const size_t b = blockIdx.y;
-    const int z = (int)(e / n), i = (int)(e % n);
-    const int l = z / g.t, r = z - l * g.t + g.E;
-    v[b * (size_t)n * n + e] = ccast<OF>(sol[b * SB + (size_t)l * strip_stride + (size_t)i * g.q + r]);
+__global__ void __launch_bounds__(256) k_scatter(StripGeom g, int L, const cpx_t<T>* __restrict__ sol,
+                                                 size_t strip_stride, size_t SB, OF* __restrict__ v) {
+    using C = cpx_t<T>;
+    __shared__ C tile[kGatherTile][kGatherTile + 1];   // [i - i0][row - r0]
+    const int q = g.q, n = g.n, t = g.t;
+    const int it = (n + kGatherTile - 1) / kGatherTile, bl = blockIdx.x / it, b = bl / L, l = bl - b * L;
+    const int i0 = (blockIdx.x - bl * it) * kGatherTile, r0 = blockIdx.y * kGatherTile;
+    sol += (size_t)b * SB + (size_t)l * strip_stride + g.E;
+    v += (size_t)b * n * n + (size_t)l * t * n;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+#pragma unroll
+    for (int u = 0; u < kGatherTile / 8; ++u) {
+        const int i = i0 + ty + 8 * u, r = r0 + tx;
+        if (i < n && r < t) tile[ty + 8 * u][tx] = sol[(size_t)i * q + r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kGatherTile / 8; ++u) {
+        const int r = r0 + ty + 8 * u, i = i0 + tx;
+        if (i < n && r < t) v[(size_t)r * n + i] = ccast<OF>(tile[tx][ty + 8 * u]);
+    }
 }
 
 // The same for the other direction's field, added to a field of this one:
 // v[i][z] = u[i][z] + (row z of the layers' solutions)[i]  (the vertical sweep's result
 // transposed back and added to the horizontal one, Algorithm 2); along z, coalesced.
+// FP32 fields are added in FP32 (the same sum as in FP64 rounded to FP32).
 template <typename T, typename AF = double2, typename OF = double2>
 __global__ void k_scatter_tadd(StripGeom g, const cpx_t<T>* __restrict__ sol, size_t strip_stride, size_t SB,
                                const AF* __restrict__ u, OF* __restrict__ v) {
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = g.n;
-    if (e >= (size_t)n * n) return;
-    const size_t b = blockIdx.y;
-    const int i = (int)(e / n), z = (int)(e % n);
+    const int n = g.n, z = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (z >= n) return;
+    const size_t b = blockIdx.z;
     const int l = z / g.t, r = z - l * g.t + g.E;
-    const size_t o = b * (size_t)n * n + e;
-    v[o] = ccast<OF>(ccast<double2>(u[o]) + ccast<double2>(sol[b * SB + (size_t)l * strip_stride + (size_t)i * g.q + r]));
+    const size_t o = (b * n + i) * (size_t)n + z;
+    const cpx_t<T> w = sol[b * SB + (size_t)l * strip_stride + (size_t)i * g.q + r];
+    if constexpr (sizeof(T) == 4 && sizeof(AF) == 8 && sizeof(OF) == 8) v[o] = u[o] + w;
+    else v[o] = ccast<OF>(ccast<double2>(u[o]) + ccast<double2>(w));
 }
 
 // natural strip layout (q rows x n, x fastest) <-> block layout (i*q + r)
@@ -833,7 +847,7 @@ int sweep_impl(ls_handle* h, int dir, const GF* g, OF* v, int nb, bool tr = fals
         if (tc) LS_TRY((sweep_tc<GF>(h, dir, g, nb, tr)));
     }
     if (!tc) {
-        const dim3 ga(gg.x, gg.y, (unsigned)(nb * L));
+        const dim3 ga(gg.x * (unsigned)(nb * L), gg.y);
         if (tr) LS_LAUNCH(h, (k_gather_all<T, true, GF>), ga, gb, 0, geo, L, g, rhs, SB);
         else LS_LAUNCH(h, (k_gather_all<T, false, GF>), ga, gb, 0, geo, L, g, rhs, SB);
         RhsSrc<T> src{};
@@ -855,13 +869,13 @@ int sweep_impl(ls_handle* h, int dir, const GF* g, OF* v, int nb, bool tr = fals
         for (int l = L - 1; l >= 0; --l) LS_TRY(layer(l, false));   // downward sweep
         for (int l = 1; l < L; ++l) LS_TRY(layer(l, true));         // upward sweep
     }
-    const size_t N = (size_t)n * n;
     if (tr && add) {
-        LS_LAUNCH(h, (k_scatter_tadd<T, AF, OF>), dim3((unsigned)((N + 255) / 256), nb), 256, 0, geo, sol, sstride, SB,
-                  add, v);
+        LS_LAUNCH(h, (k_scatter_tadd<T, AF, OF>), dim3((unsigned)((n + 255) / 256), (unsigned)n, (unsigned)nb), 256, 0,
+                  geo, sol, sstride, SB, add, v);
         return LS_OK;
     }
-    LS_LAUNCH(h, (k_scatter<T, OF>), dim3((unsigned)((N + 255) / 256), nb), 256, 0, geo, sol, sstride, SB, v);
+    LS_LAUNCH(h, (k_scatter<T, OF>), dim3(gg.x * (unsigned)(nb * L), (unsigned)((h->t + kGatherTile - 1) / kGatherTile)),
+              gb, 0, geo, L, sol, sstride, SB, v);
     return LS_OK;
 }
 
@@ -1057,7 +1071,7 @@ static int bd_direct_mixed(ls_handle* h, const float2* g, float2* v, int nb) {
     float2* u1f = reinterpret_cast<float2*>(static_cast<double2*>(h->lanes[h->lane].vtmp) + 2 * N * nb);
     float2* ef = u1f + N * nb;
     LS_TRY((sweep_impl<float, float2, float2, float2>(h, 0, g, u1f, nb)));
-    LS_TRY(ls_stencil_refine_f32(h, 0, u1f, g, ef, nb));   // e = g - C u1
+    LS_TRY(ls_stencil_refine_f32(h, u1f, g, ef, nb));   // e = g - C u1
     // vertical layers on e as it is stored (their grid is its transpose): the gather reads
     // it transposed, and the scatter writes v = u1 + the result, transposed back
     return sweep_impl<float, float2, float2, float2>(h, 1, ef, v, nb, true, u1f);
