@@ -104,15 +104,18 @@ int ls_timing_begin(ls_handle* h) {
             h->tev.push_back(e);
         }
         h->tkind.resize(h->tev.size() / 2);
+        h->tcount.resize(h->tev.size() / 2);
     }
     LS_CUDA(cudaEventRecord(h->tev[2 * h->tused], h->stream));
     return LS_OK;
 }
 
-int ls_timing_end(ls_handle* h, int kind) {
+// count: operations the interval covers (a launch that serves several members of a batch)
+int ls_timing_end(ls_handle* h, int kind, int count) {
     if (!h->timing) return LS_OK;
     LS_CUDA(cudaEventRecord(h->tev[2 * h->tused + 1], h->stream));
     h->tkind[h->tused] = kind;
+    h->tcount[h->tused] = count;
     h->tused++;
     return LS_OK;
 }
@@ -131,7 +134,7 @@ int ls_timing_collect(ls_handle* h) {
             h->n_apply64++;
         } else if (h->tkind[k] == 3) {
             h->t_stencil_ms += ms;
-            h->n_stencil++;
+            h->n_stencil += h->tcount[k];
         } else if (h->tkind[k] == 4) {
             h->t_orth_ms += ms;
             h->n_orth++;

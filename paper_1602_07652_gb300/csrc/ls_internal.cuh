@@ -295,7 +295,7 @@ struct ls_handle {
     // timing without host synchronisation: event pairs recorded during a solve and
     // read once at its end (kind 0: FP32/mixed or FP64 apply, 1: Algorithm 2, 2: FP64 refinement apply)
     std::vector<cudaEvent_t> tev;   // 2 per interval
-    std::vector<int> tkind;
+    std::vector<int> tkind, tcount;
     size_t tused = 0;
 };
 
@@ -380,13 +380,17 @@ int ls_green_table(ls_handle* h, double2** gtab_out);          // G_w on [-n, n]
 int ls_stencils_build(ls_handle* h, const double2* gtab);      // alpha, beta for both grids
 
 // stencils + vector kernels (ls_stencil.cu)
-int ls_stencil_apply(ls_handle* h, int dir, int withm, const double2* v, const double2* g, double2* y);
 int ls_transpose64(ls_handle* h, const double2* a, double2* b);
 int ls_transpose64_b(ls_handle* h, const double2* a, double2* b, int nb);
 int ls_stencil_apply64(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y);
 int ls_stencil_apply_b(ls_handle* h, int dir, int withm, const double2* v, const double2* g, double2* y, int nb);
 int ls_stencil_refine_f32(ls_handle* h, const float2* v, const float2* g, float2* y, int nb);
-int ls_stencil_apply_f32(ls_handle* h, int mode, const float2* v, float2* y);
+int ls_stencil_members(ls_handle* h, int mode, const double2* v, double2* y, const int* members, int cnt);
+int ls_stencil_members(ls_handle* h, int mode, const float2* v, float2* y, const int* members, int cnt);
+int ls_vec_scale_b(ls_handle* h, const double2* x, double2* y, size_t mstride, const int* members, int cnt,
+                   const double* a);
+int ls_vec_scale_b(ls_handle* h, const float2* x, float2* y, size_t mstride, const int* members, int cnt,
+                   const double* a);
 // Krylov vectors in FP64 (double2) or FP32 (float2); dot products summed in FP64
 // One fused pass of a Gram-Schmidt step against nvec directions (ls_stencil.cu) for
 // members members[0..cnt) of a lockstep batch in one launch (member m: V and w at

@@ -28,7 +28,7 @@
 #include "ls_internal.cuh"
 
 int ls_timing_begin(ls_handle* h);
-int ls_timing_end(ls_handle* h, int kind);
+int ls_timing_end(ls_handle* h, int kind, int count = 1);
 
 namespace {
 
@@ -83,39 +83,29 @@ int alloc_space(ls_handle* h, KrylovSpace<VT>& S, int m, int nbcap) {
     return LS_OK;
 }
 
+// y_m = op x_m for the listed members (vectors at + m * N): C as one launch for all of them, H
+// (whose transforms share one workspace) member by member.
 // FP32 vectors (LS_MIXED): H with the FP32-I/O convolution, C with the FP32 stencil
-int apply_op(ls_handle* h, Op op, const float2* x, float2* y) {
-    if (op == OP_HMIX) {
-        LS_TRY(ls_timing_begin(h));
-        LS_TRY(ls_apply32(h, x, y));
-        return ls_timing_end(h, 0);
-    }
+int apply_h(ls_handle* h, Op op, const float2* x, float2* y) {
+    return op == OP_HMIX ? ls_apply32(h, x, y) : LS_EINVAL;   // the FP64 apply takes FP64 vectors
+}
+int apply_h(ls_handle* h, Op op, const double2* x, double2* y) {
+    return op == OP_H64 ? ls_apply64(h, x, y) : ls_apply_mx(h, x, y);
+}
+template <typename VT>
+int apply_op(ls_handle* h, Op op, const VT* x, VT* y, const std::vector<int>& members) {
+    const size_t N = (size_t)h->n * h->n;
     if (op == OP_C) {
         LS_TRY(ls_timing_begin(h));
-        LS_TRY(ls_stencil_apply_f32(h, 1, x, y));
-        return ls_timing_end(h, 3);
+        LS_TRY(ls_stencil_members(h, 1, x, y, members.data(), (int)members.size()));
+        return ls_timing_end(h, 3, (int)members.size());
     }
-    return LS_EINVAL;   // the FP64 apply takes FP64 vectors
-}
-
-int apply_op(ls_handle* h, Op op, const double2* x, double2* y) {
-    switch (op) {
-        case OP_H64: {
-            LS_TRY(ls_timing_begin(h));
-            LS_TRY(ls_apply64(h, x, y));
-            return ls_timing_end(h, 0);
-        }
-        case OP_HMIX: {
-            LS_TRY(ls_timing_begin(h));
-            LS_TRY(ls_apply_mx(h, x, y));
-            return ls_timing_end(h, 0);
-        }
-        default: {
-            LS_TRY(ls_timing_begin(h));
-            LS_TRY(ls_stencil_apply(h, 0, 1, x, nullptr, y));
-            return ls_timing_end(h, 3);
-        }
+    for (int m : members) {
+        LS_TRY(ls_timing_begin(h));
+        LS_TRY(apply_h(h, op, x + m * N, y + m * N));
+        LS_TRY(ls_timing_end(h, 0));
     }
+    return LS_OK;
 }
 
 struct Result {
@@ -163,8 +153,6 @@ int gs_chunk(ls_handle* h, const float2* v, float2* z, int cnt) {
     for (int b = 0; b < cnt; ++b) LS_TRY(ls_vec_copy(h, out + b * N, z + b * N));
     return LS_OK;
 }
-int stencil_A(ls_handle* h, const double2* v, double2* y) { return ls_stencil_apply(h, 0, 0, v, nullptr, y); }
-int stencil_A(ls_handle* h, const float2* v, float2* y) { return ls_stencil_apply_f32(h, 0, v, y); }
 
 template <typename VT>
 int apply_pc_b(ls_handle* h, Pc pc, VT* v, VT* z, int nb, const unsigned char* on, ls_stats* st) {
@@ -233,12 +221,12 @@ int apply_pc_b(ls_handle* h, Pc pc, VT* v, VT* z, int nb, const unsigned char* o
     // Algorithm 3: z = GMRES(C, A v, Algorithm 2, inner_tol), all members at once
     Ctx* c = ctx_of(h);
     VT* tA = tmpA_of(c, (VT*)nullptr);
+    std::vector<int> act;
     for (int b = 0; b < top; ++b)
-        if (on[b]) {
-            LS_TRY(ls_timing_begin(h));
-            LS_TRY(stencil_A(h, v + b * N, tA + b * N));
-            LS_TRY(ls_timing_end(h, 3));
-        }
+        if (on[b]) act.push_back(b);
+    LS_TRY(ls_timing_begin(h));
+    LS_TRY(ls_stencil_members(h, 0, (const VT*)v, tA, act.data(), (int)act.size()));
+    LS_TRY(ls_timing_end(h, 3, (int)act.size()));
     std::vector<double> tl(nb, h->opts.inner_tol);
     std::vector<Result> r(nb);
     LS_TRY(fgmres_b(h, c, inner_space<VT>(c), OP_C, PC_BD, (const VT*)tA, z, false, tl.data(), h->opts.inner_maxit,
@@ -294,7 +282,7 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
         }
         nz.push_back(i);
         if (x0) {
-            LS_TRY(apply_op(h, op, xi, ri));
+            LS_TRY(apply_op(h, op, (const VT*)x, S.r, {i}));
             LS_TRY(ls_vec_axpby(h, make_double2(1, 0), bi, make_double2(-1, 0), ri));  // r = b - A x
         } else {
             LS_TRY(ls_vec_zero(h, xi));
@@ -317,20 +305,22 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
     std::vector<double2> hh_all(HS * nb);  // host copy of the members' coefficients
     std::vector<unsigned char> on(nb);
     for (;;) {
-        bool any = false;
+        std::vector<int> scaled;     // members whose next direction is scaled, and by what
+        std::vector<double> factor;
         for (int i = 0; i < nb; ++i) {
             Member& e = M[i];
             e.cyc = e.active;
             if (!e.active) continue;
-            any = true;
-            LS_TRY(ls_vec_axpby(h, make_double2(1.0 / e.beta, 0), S.r + i * N, make_double2(0, 0), V(0, i)));
+            scaled.push_back(i);
+            factor.push_back(1.0 / e.beta);
             std::fill(e.gv.begin(), e.gv.end(), cd(0));
             std::fill(e.H.begin(), e.H.end(), cd(0));
             e.gv[0] = e.beta;
             e.cyc0 = e.relres;
             e.k = 0;
         }
-        if (!any) break;
+        if (scaled.empty()) break;
+        LS_TRY(ls_vec_scale_b(h, (const VT*)S.r, V(0, 0), N, scaled.data(), (int)scaled.size(), factor.data()));
         for (int j = 0; j < m; ++j) {
             bool inc = false;
             for (int i = 0; i < nb; ++i) {
@@ -343,10 +333,8 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
             LS_TRY(apply_pc_b(h, pcj, V(j, 0), Zb(j), nb, on.data(), st));
             std::vector<int> ons;
             for (int i = 0; i < nb; ++i)
-                if (on[i]) {
-                    ons.push_back(i);
-                    LS_TRY(apply_op(h, op, Zb(j) + i * N, V(j + 1, i)));
-                }
+                if (on[i]) ons.push_back(i);
+            LS_TRY(apply_op(h, op, (const VT*)Zb(j), V(j + 1, 0), ons));
             // CGS2 against V_0..V_j in three fused passes (dots; update and dots; update and
             // norm), each one launch for all members; coefficients stay on the device
             const int cnt = (int)ons.size();
@@ -360,6 +348,8 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
             LS_CUDA(cudaMemcpyAsync(hh_all.data(), S.hdev, sizeof(double2) * HS * nb, cudaMemcpyDeviceToHost,
                                     h->stream));
             LS_CUDA(cudaStreamSynchronize(h->stream));
+            scaled.clear();
+            factor.clear();
             for (int i = 0; i < nb; ++i) {
                 if (!on[i]) continue;
                 Member& e = M[i];
@@ -399,9 +389,11 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
                     e.cyc = false;
                     continue;
                 }
-                VT* vn = V(j + 1, i);
-                LS_TRY(ls_vec_axpby(h, make_double2(1.0 / hn, 0), vn, make_double2(0, 0), vn));
+                scaled.push_back(i);
+                factor.push_back(1.0 / hn);
             }
+            LS_TRY(ls_vec_scale_b(h, (const VT*)V(j + 1, 0), V(j + 1, 0), N, scaled.data(), (int)scaled.size(),
+                                  factor.data()));
         }
         // end of the cycle: x += Z y for every member that iterated, then its true residual
         std::vector<int> done;
@@ -418,11 +410,11 @@ int fgmres_b(ls_handle* h, Ctx* c, KrylovSpace<VT>& S, Op op, Pc pc, const VT* b
             std::vector<double2> yc(k);
             for (int r = 0; r < k; ++r) yc[r] = make_double2(e.y[r].real(), e.y[r].imag());
             VT* xi = x + i * N;
-            VT* ri = S.r + i * N;
             LS_TRY(ls_vec_combine(h, k, Zb(0) + i * N, ldv, yc.data(), xi));
-            LS_TRY(apply_op(h, op, xi, ri));
-            LS_TRY(ls_vec_axpby(h, make_double2(1, 0), b + i * N, make_double2(-1, 0), ri));
         }
+        LS_TRY(apply_op(h, op, (const VT*)x, S.r, done));
+        for (int i : done)
+            LS_TRY(ls_vec_axpby(h, make_double2(1, 0), b + i * N, make_double2(-1, 0), S.r + i * N));
         LS_TRY(ls_vec_norms_b(h, (const VT*)S.r, N, done.data(), (int)done.size(), nrm.data()));
         for (int i : done) {
             Member& e = M[i];

@@ -14,7 +14,18 @@
 
 namespace {
 
-// batch member b = blockIdx.z works on v, g, y at offset b * n * n (m is shared).
+// Members of a lockstep batch that a batched vector kernel serves: grid row y works on
+// member idx[y], whose vectors start idx[y] * mstride after the block's base pointers.
+struct MemberList {
+    int idx[LS_MAX_BATCH];
+};
+MemberList first_members(int cnt) {
+    MemberList ml{};
+    for (int c = 0; c < cnt && c < LS_MAX_BATCH; ++c) ml.idx[c] = c;
+    return ml;
+}
+
+// batch member b = ml.idx[blockIdx.z] works on v, g, y at offset b * n * n (m is shared).
 // R: arithmetic type of the coefficients and the sum (FP64 I/O either way); FP32 is
 // used where the stencil only feeds the preconditioner in mixed precision (on
 // GB300 the FP64 form is bound by the FP64 units, the FP32 form by memory).
@@ -31,14 +42,14 @@ template <int MODE, typename R, typename VF = double2, typename YF = double2, ty
           typename MT = double>  // 0: y = A v  1: y = C v  2: y = g - C v
 __global__ void __launch_bounds__(256) k_stencil(int n, const StencilTables* __restrict__ tab,
                                                  const MT* __restrict__ m, const VF* __restrict__ v,
-                                                 const GF* __restrict__ g, YF* __restrict__ y) {
+                                                 const GF* __restrict__ g, YF* __restrict__ y, MemberList ml) {
     using CR = cpx_t<R>;
     constexpr int HX = kStX + 2, HZ = kStZ + 2, HN = HX * HZ;
     __shared__ CR sa[81], sb[81];
     __shared__ CR sv[HZ][HX];
     __shared__ R sm[MODE >= 1 ? HZ : 1][MODE >= 1 ? HX : 1];
     {
-        const size_t off = (size_t)blockIdx.z * n * n;
+        const size_t off = (size_t)ml.idx[blockIdx.z] * n * n;
         v += off;
         y += off;
         if (MODE == 2) g += off;
@@ -202,12 +213,6 @@ __global__ void k_update(size_t N, int nvec, const VT* __restrict__ V, size_t ld
     }
 }
 
-// Members of a lockstep batch that a batched vector kernel serves: grid row y works on
-// member idx[y], whose vectors start idx[y] * mstride after the block's base pointers.
-struct MemberList {
-    int idx[LS_MAX_BATCH];
-};
-
 // One pass of a classical Gram-Schmidt step against nvec <= G directions V_i (stride ld),
 // for the members of a batch at once, with everything that is local to an element fused
 // into the pass:
@@ -337,6 +342,22 @@ __global__ void k_axpby(size_t N, double2 a, const XT* __restrict__ x, double2 b
         y[k] = aa * ccast<YT>(x[k]) + bb * y[k];
 }
 
+struct Scales {
+    double a[LS_MAX_BATCH];
+};
+// y_m = a_m x_m for the listed members (grid row y serves member ml.idx[y] with factor sc.a[y])
+template <typename VT>
+__global__ void k_scale(size_t N, const VT* __restrict__ x, VT* __restrict__ y, size_t mstride, MemberList ml,
+                        Scales sc) {
+    using R = typename real_of<VT>::type;
+    const R a = (R)sc.a[blockIdx.y];
+    const size_t o = (size_t)ml.idx[blockIdx.y] * mstride;
+    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (size_t)gridDim.x * blockDim.x) {
+        const VT v = x[o + k];
+        y[o + k] = mkc(a * v.x, a * v.y);
+    }
+}
+
 // y = x, converting between the vector types
 template <typename XT, typename YT>
 __global__ void k_copy(size_t N, const XT* __restrict__ x, YT* __restrict__ y) {
@@ -382,58 +403,68 @@ extern "C" int ls_check_conversions(const double* d, const float* f, long long n
 }
 
 template <typename R>
-int stencil_launch(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y, int nb) {
+int stencil_launch(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y,
+                   const MemberList& ml, int cnt) {
     const int n = h->n;
-    const size_t N = (size_t)n * n;
-    (void)N;
-    const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), nb);
+    const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), (unsigned)cnt);
     const dim3 block(kStX, 256 / kStX);
     const double* m = dir == 0 ? h->m64 : h->mT64;
     const StencilTables* tab = h->dtabs + dir;
-    if (mode == 0) LS_LAUNCH(h, (k_stencil<0, R>), grid, block, 0, n, tab, m, v, g, y);
-    else if (mode == 1) LS_LAUNCH(h, (k_stencil<1, R>), grid, block, 0, n, tab, m, v, g, y);
-    else LS_LAUNCH(h, (k_stencil<2, R>), grid, block, 0, n, tab, m, v, g, y);
+    if (mode == 0) LS_LAUNCH(h, (k_stencil<0, R>), grid, block, 0, n, tab, m, v, g, y, ml);
+    else if (mode == 1) LS_LAUNCH(h, (k_stencil<1, R>), grid, block, 0, n, tab, m, v, g, y, ml);
+    else LS_LAUNCH(h, (k_stencil<2, R>), grid, block, 0, n, tab, m, v, g, y, ml);
+    return LS_OK;
+}
+// FP32 fields, medium and arithmetic
+int stencil_launch32(ls_handle* h, int mode, const float2* v, const float2* g, float2* y, const MemberList& ml,
+                     int cnt) {
+    const int n = h->n;
+    const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), (unsigned)cnt);
+    const dim3 block(kStX, 256 / kStX);
+    auto* k = mode == 0   ? k_stencil<0, float, float2, float2, float2, float>
+              : mode == 1 ? k_stencil<1, float, float2, float2, float2, float>
+                          : k_stencil<2, float, float2, float2, float2, float>;
+    LS_LAUNCH(h, k, grid, block, 0, n, h->dtabs, h->m32, v, g, y, ml);
     return LS_OK;
 }
 
 // FP64 arithmetic (the operator entry points A and C of the ABI)
 int ls_stencil_apply64(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y) {
-    return stencil_launch<double>(h, dir, mode, v, g, y, 1);
+    return stencil_launch<double>(h, dir, mode, v, g, y, first_members(1), 1);
 }
 
 // Inside the solve: FP32 arithmetic in mixed precision (the stencils feed only the
 // preconditioner, Algorithm 3 and Algorithm 2), FP64 otherwise.
 int ls_stencil_apply_b(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y, int nb) {
-    if (h->prec == LS_MIXED) return stencil_launch<float>(h, dir, mode, v, g, y, nb);
-    return stencil_launch<double>(h, dir, mode, v, g, y, nb);
+    if (h->prec == LS_MIXED) return stencil_launch<float>(h, dir, mode, v, g, y, first_members(nb), nb);
+    return stencil_launch<double>(h, dir, mode, v, g, y, first_members(nb), nb);
 }
 
 // Algorithm 2's refinement residual e = g - C u1 in mixed precision, u1 and e in FP32
 // storage (their values are FP32 either way); FP32 coefficients and sums.
 int ls_stencil_refine_f32(ls_handle* h, const float2* v, const float2* g, float2* y, int nb) {
-    const int n = h->n;
-    const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), nb);
-    const dim3 block(kStX, 256 / kStX);
-    LS_LAUNCH(h, (k_stencil<2, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, g, y);
-    return LS_OK;
+    return stencil_launch32(h, 2, v, g, y, first_members(nb), nb);
 }
 
-// y = A v (mode 0) or C v (mode 1) with FP32 vectors and FP32 arithmetic (the mixed
-// precision inner solve's operator)
-int ls_stencil_apply_f32(ls_handle* h, int mode, const float2* v, float2* y) {
-    const int n = h->n;
-    const dim3 grid((unsigned)((n + kStX - 1) / kStX), (unsigned)((n + kStZ - 1) / kStZ), 1);
-    const dim3 block(kStX, 256 / kStX);
-    const float2* none = nullptr;
-    if (mode == 0)
-        LS_LAUNCH(h, (k_stencil<0, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, none, y);
-    else
-        LS_LAUNCH(h, (k_stencil<1, float, float2, float2, float2, float>), grid, block, 0, n, h->dtabs, h->m32, v, none, y);
+// y = A v (mode 0) or C v (mode 1) for the listed members of a lockstep batch in one launch
+// (member m: v and y at + m * n * n): the inner solve's operators.
+static int members_of(const int* members, int cnt, MemberList* ml) {
+    if (cnt < 0 || cnt > LS_MAX_BATCH) return LS_EINVAL;
+    *ml = MemberList{};
+    for (int c = 0; c < cnt; ++c) ml->idx[c] = members[c];
     return LS_OK;
 }
-
-int ls_stencil_apply(ls_handle* h, int dir, int mode, const double2* v, const double2* g, double2* y) {
-    return ls_stencil_apply_b(h, dir, mode, v, g, y, 1);
+int ls_stencil_members(ls_handle* h, int mode, const double2* v, double2* y, const int* members, int cnt) {
+    MemberList ml;
+    LS_TRY(members_of(members, cnt, &ml));
+    if (cnt == 0) return LS_OK;
+    return h->prec == LS_MIXED ? stencil_launch<float>(h, 0, mode, v, nullptr, y, ml, cnt)
+                               : stencil_launch<double>(h, 0, mode, v, nullptr, y, ml, cnt);
+}
+int ls_stencil_members(ls_handle* h, int mode, const float2* v, float2* y, const int* members, int cnt) {
+    MemberList ml;
+    LS_TRY(members_of(members, cnt, &ml));
+    return cnt == 0 ? LS_OK : stencil_launch32(h, mode, v, nullptr, y, ml, cnt);
 }
 
 int ls_transpose64_b(ls_handle* h, const double2* a, double2* b, int nb) {
@@ -540,7 +571,10 @@ int vec_orth_b(ls_handle* h, int mode, int nvec, const VT* V, size_t ld, size_t 
     }
     MemberList ml;
     for (int c = 0; c < cnt; ++c) ml.idx[c] = members[c];
-    const int bpm = RED_BLOCKS / cnt;   // >= 9: cnt <= LS_MAX_BATCH
+    // blocks per member: RED_BLOCKS shared out, and no more than 1024 elements each need (a 64^2
+    // member is 4 blocks, not 608 whose partial sums the final kernel would add)
+    const size_t need = (N + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+    const int bpm = need < (size_t)(RED_BLOCKS / cnt) ? (int)need : RED_BLOCKS / cnt;
     const dim3 grid((unsigned)bpm, (unsigned)cnt);
     LS_TRY(red_reserve(h, (size_t)RED_BLOCKS * 64 + 256));
     double2* partial = reinterpret_cast<double2*>(h->red);
@@ -588,6 +622,28 @@ int ls_vec_norms_b(ls_handle* h, const double2* w, size_t mstride, const int* me
 }
 int ls_vec_norms_b(ls_handle* h, const float2* w, size_t mstride, const int* members, int cnt, double* out) {
     return vec_norms_b(h, w, mstride, members, cnt, out);
+}
+
+// y_m = a_m x_m for the members members[0..cnt) of a batch in one launch (in place if x == y)
+template <typename VT>
+static int vec_scale_b(ls_handle* h, const VT* x, VT* y, size_t mstride, const int* members, int cnt, const double* a) {
+    MemberList ml;
+    LS_TRY(members_of(members, cnt, &ml));
+    if (cnt == 0) return LS_OK;
+    Scales sc{};
+    for (int c = 0; c < cnt; ++c) sc.a[c] = a[c];
+    const size_t N = (size_t)h->n * h->n;
+    const unsigned gx = (unsigned)((N + 1023) / 1024), cap = (unsigned)(4 * RED_BLOCKS / cnt);
+    LS_LAUNCH(h, k_scale<VT>, dim3(gx < cap ? gx : cap, (unsigned)cnt), 256, 0, N, x, y, mstride, ml, sc);
+    return LS_OK;
+}
+int ls_vec_scale_b(ls_handle* h, const double2* x, double2* y, size_t mstride, const int* members, int cnt,
+                   const double* a) {
+    return vec_scale_b(h, x, y, mstride, members, cnt, a);
+}
+int ls_vec_scale_b(ls_handle* h, const float2* x, float2* y, size_t mstride, const int* members, int cnt,
+                   const double* a) {
+    return vec_scale_b(h, x, y, mstride, members, cnt, a);
 }
 
 int ls_vec_combine(ls_handle* h, int nvec, const double2* Z, size_t ld, const double2* coef_host, double2* x) {
