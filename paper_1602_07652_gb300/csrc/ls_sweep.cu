@@ -892,7 +892,10 @@ int smem_optin_modes(int q) {
 }
 template <typename T, int NB>
 int smem_optin_nb(int q) { return smem_optin_modes<T, NB, 0, 1, 2, 4, 5, 6>(q); }
-int smem_optin(bool mixed, int q) {
+// (a kernel's limit is the process's, not the handle's: always that of the tallest strip, so that
+// a handle of shorter strips does not lower it under another one)
+int smem_optin(bool mixed) {
+    constexpr int q = 112;
     if (mixed) {
         LS_TRY((smem_optin_nb<float, 1>(q)));
         LS_TRY((smem_optin_nb<float, 2>(q)));
@@ -1032,7 +1035,7 @@ int ls_cr_inverse_build(ls_handle* h, int dir) {
 }
 
 int ls_sweep_alloc(ls_handle* h) {
-    LS_TRY(smem_optin(h->prec == LS_MIXED, h->q));
+    LS_TRY(smem_optin(h->prec == LS_MIXED));
     for (int k = 1; k < ls_handle::kLanes; ++k) {
         LS_CUDA(cudaStreamCreateWithFlags(&h->lanes[k].stream, cudaStreamNonBlocking));
         LS_CUDA(cudaEventCreateWithFlags(&h->lanes[k].done, cudaEventDisableTiming));

@@ -62,3 +62,21 @@ def test_local_solves_and_batches_match_oracle(n, L, E, prec, tol):
                 for b in range(nb):
                     assert rel(v[b], bd(g[b])) < tol, (split, nb, b)
     s.close()
+
+
+def test_a_handle_of_shorter_strips_leaves_a_taller_one_its_shared_memory():
+    # q = 112, then handles of q = 104 and 100 on the same kernels: in batches of 8 all ask for
+    # more than 48 KB a CTA, the first for the most
+    n = 200
+    w = inputs.omega_for_ppw(n, 10.0)
+    m = cuda(inputs.bump_medium(n, nbumps=4, seed=3))
+    s = binding.Solver(m, w, layers=2, ext=6, precision=binding.LS_MIXED)
+    s.ls_factor()
+    s.ls_set_tensor_steps(0)
+    g = cuda(np.stack([inputs.random_field(n, 70 + b) for b in range(8)]))
+    alone = s.ls_precond_bd_batch(g).cpu()
+    others = [binding.Solver(m, w, layers=2, ext=2, precision=binding.LS_MIXED),
+              binding.Solver(m[:180, :180].contiguous(), w, layers=2, ext=5, precision=binding.LS_MIXED)]
+    assert torch.equal(s.ls_precond_bd_batch(g).cpu(), alone)
+    for o in others + [s]:
+        o.close()
