@@ -233,13 +233,13 @@ int ls_solve_group(int nprob, ls_handle* const* hs, const ls_c64* const* f, doub
  *     HBM and shared memory by TMA; 8 = shape 6 with the two columns of a tile in
  *     packed FP32x2 instructions (4 needs 32 <= P <= 4096, 0 and the other shapes but
  *     1 need 256 <= P <= 4096); 1 = the generic radix-8 transforms on 4-column tiles.  A
- *     handle starts with 4 up to P = 512 and with 8 above;
+ *     handle starts with 4 up to P = 512, 2 at 1024, 6 at 2048 and 8 at 4096;
  *   - the band-block batching of Algorithm 2 for nrhs right-hand sides: bd_chunk
  *     = right-hand sides per pass over the local-solve factors (1, 2, 4, 8;
  *     FP64 up to 4), chunks running concurrently on separate streams, and
  *     cr_split = whether the block-cyclic-reduction steps of levels with few
- *     blocks split each block over several CTAs (partial sums combined in a
- *     fixed order, so results are reproducible for a given choice).
+ *     blocks split each block's rows over several CTAs (sums in a fixed order,
+ *     so results are reproducible for a given choice).
  * Each candidate runs once, then reps times under CUDA events; the fastest is
  * kept by the handle for later applies and batched solves (results agree up to
  * rounding whichever is chosen).  Before ls_factor only the FFT shape is tuned
@@ -251,8 +251,8 @@ typedef struct {
     double fft_ms[9];   /* LS-apply (FP64 I/O, FP32 arithmetic) per variant; -1: n/a   */
     double bd_ms[4];    /* Algorithm 2 ms per right-hand side, chunks 1, 2, 4, 8 (0: not tried) */
     double bd_ms_nosplit[4]; /* the same without splitting the blocks of small levels        */
-    int cr_split;       /* 1: the reduction steps of levels with fewer blocks than SMs split
-                           each block's columns over several CTAs; 0: one CTA per block     */
+    int cr_split;       /* 1: the CUDA-core reduction steps of levels with few blocks split
+                           each block's rows over several CTAs; 0: one CTA per block        */
     double bd_ms_tc[4]; /* LS_MIXED: the same with the reduction steps on the tensor cores,
                            chunks 1, 8, 16, 32 (0: not tried; tried only while that form
                            is switched on, see ls_set_tensor_steps)                        */
@@ -326,8 +326,8 @@ int ls_set_double_float(ls_handle* h, int on);
 int ls_set_reduced_inverse(ls_handle* h, int on);
 
 /* ls_set_reduction -- pin the form of the block-cyclic-reduction local solves of
- * Algorithm 1 (Sec. 3.4): cr_split 1 lets the steps of levels with fewer blocks
- * than SMs split each block's columns over several CTAs, 0 keeps one CTA per block
+ * Algorithm 1 (Sec. 3.4): cr_split 1 lets the CUDA-core steps of levels with few
+ * blocks split each block's rows over several CTAs, 0 keeps one CTA per block
  * (as in ls_tuning).  Synchronises the handle's stream and drops the captured sweep
  * graphs when the form changes.  LS_EINVAL for other values.  Results agree up to
  * rounding in either form. */

@@ -827,11 +827,13 @@ bool ls_fft16_supported(const ls_handle* h, int shape) {
     return shape != 1 && h->lp >= (shape == 4 ? 5 : 8) && h->lp <= 12;
 }
 
-// The shape a handle starts with: radix-8 1-column tiles up to P = 512 (n = 128: 9.1 us on the
-// device against 11.4 with 2-column radix-16 tiles, 256: 10.3 against 15.4), TMA tiles in
-// packed FP32x2 arithmetic above (512: 16.0 against 16.4, 1024: 43.3 against 51.7, 2048: 139
-// against 191).
-int ls_fft16_default(const ls_handle* h) { return h->lp <= 9 ? 4 : 8; }
+// The shape a handle starts with, by length (back-to-back calls, us): radix-8 1-column tiles up
+// to P = 512 (n = 128: 6.2 against 8.1 with 2-column radix-16 tiles, 256: 8.2 against 10.3);
+// 2-column radix-16 tiles at P = 1024, moved by threads (n = 400: 12.7 against 13.5 by TMA, 512:
+// 13.7 against 13.9), and at P = 2048, moved by TMA (800: 34.6 against 35.3 by threads and 35.5
+// packed, 1024: 36.8, 39.9 and 37.3); by TMA in packed FP32x2 arithmetic at P = 4096 (1600: 106.5
+// against 110.5 unpacked, 2048: 122.6 against 125.8).
+int ls_fft16_default(const ls_handle* h) { return h->lp <= 9 ? 4 : (h->lp == 10 ? 2 : (h->lp == 11 ? 6 : 8)); }
 
 int ls_fft16_init(ls_handle* h) {
     if (h->lp >= 8 && h->lp <= 12) {
