@@ -111,7 +111,7 @@ struct SrcIncDf {
     int n;
     template <typename C>
     __device__ __forceinline__ C load(int z, int x) const {
-        return ccast<C>(m[(size_t)z * n + x] * (ldg_c(&ex[x]) * ldg_c(&ez[z])));
+        return ccast<C>(m[(size_t)z * n + x] * (ex[x] * ez[z]));
     }
 };
 

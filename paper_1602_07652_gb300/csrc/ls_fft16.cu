@@ -650,8 +650,8 @@ __global__ void __launch_bounds__(Geo<LP, LE, kTmaCta>::THREADS, MINB) k_cols16_
 // (each thread fetches the elements it will write), so its latency hides behind the
 // last stage, and the CTA needs no shared memory beyond the exchange buffer.
 template <int LP, typename UIO>
-__global__ void __launch_bounds__(Geo<LP, 4>::THREADS, 4) k_rows16_inv(int nrows, int n, const float2* __restrict__ X,
-                                                                    const UIO* __restrict__ u, UIO* __restrict__ y,
+__global__ void __launch_bounds__(Geo<LP, 4>::THREADS, 4) k_rows16_inv(int nrows, int n, const float2* X,
+                                                                    const UIO* u, UIO* y,
                                                                     const float2* __restrict__ tw) {
     using Gm = Geo<LP, 4>;
     constexpr int P = Gm::P, T = Gm::T, E = Gm::E, R = 1 << Gm::LRL;

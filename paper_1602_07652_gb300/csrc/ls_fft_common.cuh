@@ -72,6 +72,8 @@ __device__ __forceinline__ void dft_reg(C* v) {
 }
 
 // ---------------------------------------------------------------- pass-1 sources
+// The fields and factors that an earlier kernel of the stream writes (u, ex, ez) are read with
+// ordinary loads: a row pass may be resident while that kernel runs (pdl_wait).
 template <typename T, typename UIn>
 struct SrcMU {  // m u  (Sec. 2: D u)
     const T* m;
@@ -80,7 +82,7 @@ struct SrcMU {  // m u  (Sec. 2: D u)
     template <typename C>
     __device__ __forceinline__ C load(int z, int x) const {
         const size_t i = (size_t)z * n + x;
-        return m[i] * hw_cast<C>(__ldg(&u[i]));
+        return m[i] * hw_cast<C>(u[i]);
     }
 };
 
@@ -92,7 +94,7 @@ struct SrcInc {  // m u_I, u_I = exp(i w x cos) exp(i w z sin)  (Sec. 2: D u_I)
     int n;
     template <typename C>
     __device__ __forceinline__ C load(int z, int x) const {
-        const double2 ui = __ldg(&ex[x]) * __ldg(&ez[z]);
+        const double2 ui = ex[x] * ez[z];
         return m[(size_t)z * n + x] * ccast<C>(ui);
     }
 };

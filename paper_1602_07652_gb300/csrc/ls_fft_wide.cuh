@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_cols
 }
 
 template <int LP, typename C, typename W, class Dst>
-__global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows_inv(int n, const C* __restrict__ X, Dst dst,
+__global__ void __launch_bounds__(GeoW<LP>::THREADS, GeoW<LP>::MINB) k_wide_rows_inv(int n, const C* X, Dst dst,
                                                                                  const W* __restrict__ tw) {
     using Gm = GeoW<LP>;
     constexpr int T = Gm::T, R = 1 << Gm::LRL;

@@ -329,6 +329,10 @@ int ls_cuda_fail(cudaError_t e);
 // writes are visible -- it may touch only data that no kernel still in flight writes (the
 // factors and tables of ls_factor).  Every kernel of such a chain calls pdl_wait, so a
 // completed predecessor implies that everything before it has completed too.
+// What a predecessor writes is read after pdl_wait and with ordinary loads, never through the
+// read-only path (__ldg, ldg_c, a const __restrict__ parameter): that path is for memory that
+// nothing writes while the kernel is resident, and the kernel is resident before pdl_wait; the
+// compiler may move such a load above the wait, and the load need not see the new value.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
