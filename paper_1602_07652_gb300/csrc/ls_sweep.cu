@@ -105,13 +105,12 @@ struct Couple {
 // chunks a block) for NB (>= nb) batch members:
 //   out_b = base_b + sum_t M_t v_{t,b}
 //   MODE 0 (level 0 odd):     x_j = D^{-1} b_j
-//   MODE 1 (forward, k >= 2): even j: x_j = x_j - F x_{j-1} - G x_{j+1};  odd j: y_j = D^{-1} x_j
-//   MODE 5 (forward, k = 1):  the same with the level-0 even update b'_i = b_i - W_i y_{i-1}
-//          - E_i y_{i+1} formed as the blocks are read (it is never stored)
+//   MODE 1 (forward, k >= 1): even j: x_j = x_j - F x_{j-1} - G x_{j+1};  odd j: y_j = D^{-1} x_j
 //   MODE 2 (backward):        x_j = y_j - P x_{j-1} - Q x_{j+1}   (odd j, levels >= 1)
 //   MODE 3 (top block):       x_0 = D^{-1} x_0   (S = 1; only to build the reduced inverse)
 //   MODE 4 (level 0 back):    x_j = x_j - D^{-1} (W_j x_{j-1} + E_j x_{j+1})   (odd j)
 //   MODE 6 (level c):         x = S_c^{-1} y over all nc unknowns of the level
+// (the even blocks of level 0: k_cr_even)
 //
 // What bounds a step is latency: a local solve is a chain of dependent steps, most over a few
 // blocks.  On GB300 a chain of trivial kernels takes 1.0 us a link, and handing partial sums
@@ -138,7 +137,7 @@ struct CrStep {
     using C = cpx_t<T>;
     int q, k, nk;                  // strip height, level, blocks of the level
     int S, R;                      // row chunks per block (MODE 6: in all), rows of a chunk
-    int nlead;                     // MODE 1, 5: CTAs on even blocks (the odd blocks' follow)
+    int nlead;                     // MODE 1: CTAs on even blocks (the odd blocks' follow)
     const C* pool;                 // first matrix of the strip (q x q, column-major)
     size_t off_a, off_b, off_c;    // level offsets (matrices): D^{-1}; F or P; G or Q
     C* x;                          // strip vectors; member b at + b * SB
@@ -146,39 +145,38 @@ struct CrStep {
     size_t SB, YB;                 // member strides
     size_t pool_strip, x_strip;    // strip blockIdx.y (elements; the set-up runs all strips at once)
     int nb;
-    bool to_y;                     // MODE 1, 5: the even results go to y (the last level before c)
+    bool to_y;                     // MODE 1: the even results go to y (the last level before c)
     const C* inv;                  // MODE 6: S_c^{-1} (nc x nc, column-major), blocks j << c
     int nc, c;
-    RhsSrc<T> src;                 // MODE 0, 5
-    Couple<T> cp;                  // MODE 4, 5
+    RhsSrc<T> src;                 // MODE 0, k_cr_even
+    Couple<T> cp;                  // MODE 4, k_cr_even
 };
 
-template <int MODE> constexpr int cr_mats() { return MODE == 1 || MODE == 2 || MODE == 5 ? 2 : 1; }   // matrices
-template <int MODE> constexpr int cr_vecs() { return MODE == 5 ? 3 : cr_mats<MODE>(); }                // vectors
-template <int MODE> constexpr int cr_tabs() { return MODE == 5 ? 3 : (MODE == 4 ? 1 : 0); }            // coupling tables
+template <int MODE> constexpr int cr_mats() { return MODE == 1 || MODE == 2 ? 2 : 1; }   // matrices, a vector each
+template <int MODE> constexpr int cr_tabs() { return MODE == 4 ? 1 : 0; }                // coupling tables
 // columns a thread keeps in flight: 24 (FP64 32) registers of matrix entries, so that (FP32) four CTAs
 // share an SM: 768^2, one member, 71 us a solve against 80 with 40 registers, 78 with five
 // CTAs of 48 and 89 with three of 80
-template <typename T, int MODE> constexpr int cr_prefetch() { return (sizeof(T) == 8 ? 8 : 12) / cr_mats<MODE>() - (MODE == 5 ? 1 : 0); }
+template <typename T, int MODE> constexpr int cr_prefetch() { return (sizeof(T) == 8 ? 8 : 12) / cr_mats<MODE>(); }
 template <typename T, int NB> constexpr int cr_min_ctas() { return sizeof(T) == 8 ? (NB <= 2 ? 3 : 2) : (NB <= 4 ? 4 : 3); }
 // shared memory: vectors (q or nc long) | partial sums | couplings
 template <typename T, int MODE, int NB>
 constexpr size_t cr_smem(int q, int nc) {
-    return sizeof(cpx_t<T>) * ((size_t)cr_vecs<MODE>() * NB * (MODE == 6 ? nc : q) + (size_t)kMvThreads * NB +
+    return sizeof(cpx_t<T>) * ((size_t)cr_mats<MODE>() * NB * (MODE == 6 ? nc : q) + (size_t)kMvThreads * NB +
                                (size_t)cr_tabs<MODE>() * 6 * q);
 }
 
 template <typename T, int MODE, int NB>
 __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(CrStep<T> a) {
     using C = cpx_t<T>;
-    constexpr int NM = cr_mats<MODE>(), NV = cr_vecs<MODE>(), PF = cr_prefetch<T, MODE>();
+    constexpr int NM = cr_mats<MODE>(), PF = cr_prefetch<T, MODE>();
     constexpr bool kEarly = sizeof(T) == 4 && NB == 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (kEarly) pdl_trigger();
-    const int q = a.q, n = a.src.n, ncol = MODE == 6 ? a.nc : q;
-    C* vin = reinterpret_cast<C*>(smem_raw);     // [NV][NB][ncol]
-    C* red = vin + (size_t)NV * NB * ncol;       // [CG][NB][R]
-    C* tab = red + kMvThreads * NB;              // MODE 4, 5: [v][W, E][dz+1][q]
+    const int q = a.q, ncol = MODE == 6 ? a.nc : q;
+    C* vin = reinterpret_cast<C*>(smem_raw);     // [NM][NB][ncol]
+    C* red = vin + (size_t)NM * NB * ncol;       // [CG][NB][R]
+    C* tab = red + kMvThreads * NB;              // MODE 4: [W, E][dz+1][q]
     const int tid = threadIdx.x;
     const int b0 = blockIdx.z * NB, nb = a.nb - b0 < NB ? a.nb - b0 : NB;
     const C* pool = a.pool + blockIdx.y * a.pool_strip;
@@ -189,7 +187,7 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     const size_t s = (size_t)q << a.k;           // elements between neighbouring blocks of the level
     bool odd = MODE == 0 || MODE == 2 || MODE == 4;
     int bid = blockIdx.x;
-    if ((MODE == 1 || MODE == 5) && bid >= a.nlead) {
+    if (MODE == 1 && bid >= a.nlead) {
         odd = true;
         bid -= a.nlead;
     }
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     const int j = 2 * idx + (odd ? 1 : 0);
     const bool hw = j >= 1, he = j + 1 < a.nk;
     const C* Ms[NM];
-    int vb[NV], nm = 1, nv = 1;                  // the vectors' blocks (level index), matrices, vectors
+    int vb[NM], nm = 1;                          // the vectors' blocks (level index), matrices present
     if (MODE == 6) {
         Ms[0] = a.inv;
         vb[0] = 0;
@@ -209,13 +207,9 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
         const C* M1 = pool + (a.off_c + idx) * qq;
         Ms[0] = hw ? M0 : M1;
         vb[0] = hw ? j - 1 : j + 1;
-        nm = nv = (hw && he) ? 2 : 1;
+        nm = (hw && he) ? 2 : 1;
         Ms[NM - 1] = nm == 2 ? M1 : Ms[0];
         vb[NM - 1] = nm == 2 ? j + 1 : vb[0];
-        if (MODE == 5) {
-            vb[NV - 1] = j;                      // the even update of the block itself, in slot 2
-            nv = 3;
-        }
     }
     const int R = a.R, r0 = sp * R, nr = (MODE == 6 ? a.nc : q) - r0 < R ? (MODE == 6 ? a.nc : q) - r0 : R;
     const int CG = kMvThreads / R, cg = tid / R, rr = tid - cg * R;
@@ -229,12 +223,8 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
 #pragma unroll
     for (int u = 0; u < PF; ++u) load_col(pre[u], cg + u * CG);
     if constexpr (cr_tabs<MODE>() > 0) {
-        for (int e = tid; e < cr_tabs<MODE>() * 6 * q; e += kMvThreads) {
-            const int v = e / (6 * q), w = e - v * 6 * q;
-            const bool use = MODE == 4 || (v < NM ? v < nm : nv == 3);
-            const size_t i = MODE == 4 ? (size_t)j : 2 * (size_t)(v == 0 ? vb[0] : (v == 1 ? vb[NM - 1] : j));
-            if (use) tab[e] = __ldg(w < 3 * q ? &a.cp.cw[i * 3 * q + w] : &a.cp.ce[i * 3 * q + (w - 3 * q)]);
-        }
+        for (int w = tid; w < 6 * q; w += kMvThreads)
+            tab[w] = __ldg(w < 3 * q ? &a.cp.cw[(size_t)j * 3 * q + w] : &a.cp.ce[(size_t)j * 3 * q + (w - 3 * q)]);
         __syncthreads();
     }
     pdl_wait();
@@ -254,15 +244,15 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     } else {
         const int r = tid & 127;
 #pragma unroll
-        for (int p = 0; p < NV * NB; ++p) {
+        for (int p = 0; p < NM * NB; ++p) {
             const int v = p / NB, b = p % NB;
             if ((p & 1) != (tid >> 7) || r >= q) continue;
             C val = czero<C>();
-            if (b < nb && (v < nm || (MODE == 5 && v == 2 && nv == 3))) {
+            if (b < nb && v < nm) {
                 const C* xb = x + (size_t)b * a.SB;
                 if (MODE == 0) val = a.src.load(j, r, b0 + b);
                 if (MODE == 1 || MODE == 2 || MODE == 3) {
-                    val = xb[(size_t)vb[v < NM ? v : 0] * s + r];
+                    val = xb[(size_t)vb[v] * s + r];
                     if (MODE == 2 || !(odd || MODE == 3)) val = -val;
                 }
                 if (MODE == 4) {   // -(W x_{j-1} + E x_{j+1})
@@ -275,24 +265,11 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
                     }
                     val = -val;
                 }
-                if (MODE == 5) {   // b' of level-0 block i
-                    const int i = 2 * vb[v];
-                    const C* tv = tab + (size_t)v * 6 * q;
-                    val = a.src.load(i, r, b0 + b);
-#pragma unroll
-                    for (int dz = -1; dz <= 1; ++dz) {
-                        const int rz = r + dz;
-                        if (rz < 0 || rz >= q) continue;
-                        if (i >= 1) val = cfms(tv[(dz + 1) * q + r], xb[(size_t)(i - 1) * q + rz], val);
-                        if (i + 1 < n) val = cfms(tv[(dz + 4) * q + r], xb[(size_t)(i + 1) * q + rz], val);
-                    }
-                    if (!odd && v < 2) val = -val;
-                }
             }
             vin[(size_t)p * q + r] = val;
             if (kSparse) nonzero = nonzero || val.x != T(0) || val.y != T(0);
         }
-        if ((MODE == 0 || MODE == 5) && sp == 0 && tid < nb) a.src.keep_trace(MODE == 0 ? j : 2 * j, b0 + tid);
+        if (MODE == 0 && sp == 0 && tid < nb) a.src.keep_trace(j, b0 + tid);
     }
     // what the result is added to (the first of this thread's outputs: fetched ahead)
     const int nout = nb * nr;
@@ -358,12 +335,12 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
         if (MODE == 6) {
             const int jb = r / q;
             xb[(((size_t)jb << a.c) - jb) * q + r] = sum;
-        } else if (MODE == 1 || MODE == 5) {
+        } else if (MODE == 1) {
             const size_t e = (size_t)j * s + r;
             if (odd) {
                 yb[e] = sum;
             } else {
-                sum = (MODE == 5 ? vin[((size_t)2 * NB + b) * q + r] : base) + sum;
+                sum = base + sum;
                 if (a.to_y) yb[e] = sum;
                 else xb[e] = sum;
             }
@@ -375,10 +352,12 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     }
 }
 
-// Level-0 even blocks on their own (FP64): x_i = b_i - W_i y_{i-1} - E_i y_{i+1}, one thread per
-// row and member.  MODE 5 forms this up to three times per block and once per row chunk, which
-// FP32 does not notice; on the FP64 pipe it cost 7 us of a 150 us solve (400^2, q = 70), this
-// kernel about 2.
+// Level-0 even blocks: x_i = b_i - W_i y_{i-1} - E_i y_{i+1}, one thread per row and member.  A
+// link of its own in the chain, of about 2 us.  Formed where level 1 reads the blocks instead, it
+// is computed up to three times per block, again in every row chunk and for every member, and its
+// tables take shared memory: a field of Algorithm 2 on FP32 steps, that form -> this one, ms:
+// 768^2 3.42 -> 3.33 (one field), 1.99 -> 1.83 (a batch of 2), 1.12 -> 0.96 (8); 32 fields of
+// 2048^2 in chunks of 8 on four streams 4.66 -> 3.44.
 template <typename T>
 __global__ void __launch_bounds__(128) k_cr_even(CrStep<T> a) {
     const int i = 2 * blockIdx.x, b = blockIdx.y, q = a.q, n = a.src.n;
@@ -713,13 +692,8 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
         const unsigned grid = level(k, F.lev[k].nk);
         a.off_b = F.lev[k].off_f;
         a.off_c = F.lev[k].off_g;
-        if (sizeof(T) == 4 && k == 1) {
-            LS_TRY((cr_launch<T, 5, NB>(h, a, grid)));
-            continue;
-        }
-        if (k == 1)
-            LS_TRY(ls_launch_pdl(h, k_cr_even<T>, dim3((unsigned)l0.neven, (unsigned)nb), dim3(128), 0, a));
-         LS_TRY((cr_launch<T, 1, NB>(h, a, grid)));
+        if (k == 1) LS_TRY(ls_launch_pdl(h, k_cr_even<T>, dim3((unsigned)l0.neven, (unsigned)nb), dim3(128), 0, a));
+        LS_TRY((cr_launch<T, 1, NB>(h, a, grid)));
     }
     cr_split(h, a, a.nc, 1, sizeof(T) == 8 ? 4 : 8);
     LS_TRY((cr_launch<T, 6, NB>(h, a, (unsigned)a.S)));
@@ -891,7 +865,7 @@ int smem_optin_modes(int q) {
     return LS_OK;
 }
 template <typename T, int NB>
-int smem_optin_nb(int q) { return smem_optin_modes<T, NB, 0, 1, 2, 4, 5, 6>(q); }
+int smem_optin_nb(int q) { return smem_optin_modes<T, NB, 0, 1, 2, 4, 6>(q); }
 // (a kernel's limit is the process's, not the handle's: always that of the tallest strip, so that
 // a handle of shorter strips does not lower it under another one)
 int smem_optin(bool mixed) {
