@@ -252,7 +252,8 @@ typedef struct {
     double bd_ms[4];    /* Algorithm 2 ms per right-hand side, chunks 1, 2, 4, 8 (0: not tried) */
     double bd_ms_nosplit[4]; /* the same without splitting the blocks of small levels        */
     int cr_split;       /* 1: the CUDA-core reduction steps of levels with few blocks split
-                           each block's rows over several CTAs; 0: one CTA per block        */
+                           each block's rows over several CTAs; 0: one CTA per block
+                           (the reduced inverse of the last levels is split either way)     */
     double bd_ms_tc[4]; /* LS_MIXED: the same with the reduction steps on the tensor cores,
                            chunks 1, 8, 16, 32 (0: not tried; tried only while that form
                            is switched on, see ls_set_tensor_steps)                        */
@@ -328,9 +329,9 @@ int ls_set_reduced_inverse(ls_handle* h, int on);
 /* ls_set_reduction -- pin the form of the block-cyclic-reduction local solves of
  * Algorithm 1 (Sec. 3.4): cr_split 1 lets the CUDA-core steps of levels with few
  * blocks split each block's rows over several CTAs, 0 keeps one CTA per block
- * (as in ls_tuning).  Synchronises the handle's stream and drops the captured sweep
- * graphs when the form changes.  LS_EINVAL for other values.  Results agree up to
- * rounding in either form. */
+ * (as in ls_tuning; the reduced inverse of the last levels is split either way).
+ * Synchronises the handle's stream and drops the captured sweep graphs when the form
+ * changes.  LS_EINVAL for other values.  Results agree up to rounding in either form. */
 int ls_set_reduction(ls_handle* h, int cr_split);
 
 /* ls_device_timeouts -- health counter of the kernels fed by TMA (the paper has no

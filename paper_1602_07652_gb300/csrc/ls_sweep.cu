@@ -628,14 +628,16 @@ __global__ void k_strip_out(int n, int q, const cpx_t<T>* __restrict__ x, double
 StripGeom geom_of(const ls_handle* h) { return StripGeom{h->n, h->t, h->E, h->q, h->opts.shift / h->omega}; }
 
 // Row chunks per block of a reduction step: levels with few blocks are split until about
-// kCtas CTAs run, down to chunks of 8 rows (64 contiguous bytes of an FP32 column; 4 rows of
-// the reduced inverse in FP64).  FP64 steps are bound by the FP64 pipe of each SM, so they
-// are cut finer, for balance: one CTA per block left SMs with twice the others' work.  The
-// handle's cr_split switches the splitting off (1 CTA per block).
+// kCtas CTAs run, down to chunks of min_rows: 8 rows (64 contiguous bytes of an FP32 column), and
+// 4 of the reduced inverse in FP64, whose few rows would leave FP64 pipes idle.  The handle's
+// cr_split switches the splitting of the levels off (1 CTA per block); the reduced inverse is one
+// product of up to 700 rows, not a block, and is always split: on the three CTAs that its rows
+// need at least, it was the longest step of the solve (unsplit levels, a field of Algorithm 2, ms:
+// 64^2 FP64 2.47 -> 0.52, 400^2 FP64 10.7 -> 6.9, 256^2 FP32 1.80 -> 1.01).
 template <typename T>
-void cr_split(const ls_handle* h, CrStep<T>& a, int rows, int blocks, int min_rows = 8) {
+void cr_split(CrStep<T>& a, int rows, int blocks, int min_rows, bool split) {
     constexpr int kCtas = 608;
-    int S = h->cr_split ? kCtas / blocks : 1;
+    int S = split ? kCtas / blocks : 1;
     if (S > rows / min_rows) S = rows / min_rows;
     if (S < (rows + kMvThreads - 1) / kMvThreads) S = (rows + kMvThreads - 1) / kMvThreads;   // R <= kMvThreads
     a.R = (rows + S - 1) / S;
@@ -683,7 +685,7 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
         a.nk = lv.nk;
         a.off_a = lv.off_dinv;
         a.to_y = k == a.c - 1;
-        cr_split(h, a, q, blocks);
+        cr_split(a, q, blocks, 8, h->cr_split != 0);
         a.nlead = lv.neven * a.S;
         return (unsigned)(blocks * a.S);
     };
@@ -695,7 +697,7 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
         if (k == 1) LS_TRY(ls_launch_pdl(h, k_cr_even<T>, dim3((unsigned)l0.neven, (unsigned)nb), dim3(128), 0, a));
         LS_TRY((cr_launch<T, 1, NB>(h, a, grid)));
     }
-    cr_split(h, a, a.nc, 1, sizeof(T) == 8 ? 4 : 8);
+    cr_split(a, a.nc, 1, sizeof(T) == 8 ? 4 : 8, true);
     LS_TRY((cr_launch<T, 6, NB>(h, a, (unsigned)a.S)));
     for (int k = a.c - 1; k >= 1; --k) {
         if (!F.lev[k].nodd) continue;
