@@ -239,7 +239,7 @@ struct ls_handle {
     DirFactors fac[2];
     // Sweep workspaces ("lanes"): every lane holds the strip right-hand sides and
     // solutions, traces, transpose scratch, Algorithm 2 staging buffers and its CUDA
-    // graphs (one per batch size) for up to nb_cap right-hand sides, so that chunks
+    // graphs (one per batch size and share of the chip) for up to nb_cap right-hand sides, so that chunks
     // of a batch can run their Algorithm 2 chains concurrently on different streams.
     struct SweepLane {
         void* srhs = nullptr;      // every strip's right-hand side (n*q each), nb_cap sets
@@ -248,9 +248,12 @@ struct ls_handle {
         void* vtmp = nullptr;      // 4 n*n complex scratch fields (FP64) per right-hand side
         double2* bd_in = nullptr;  // graph staging
         double2* bd_out = nullptr;
-        cudaGraph_t graph[kMaxBatch + 1] = {};
-        cudaGraphExec_t exec[kMaxBatch + 1] = {};
-        long long nodes[kMaxBatch + 1] = {};
+        struct Graph {
+            cudaGraph_t graph = nullptr;
+            cudaGraphExec_t exec = nullptr;
+            long long nodes = 0;
+        };
+        Graph graphs[kMaxBatch + 1][3];
         int nb_cap = 0;
         void* cr_y = nullptr;           // y_j of a local solve's odd blocks (CUDA-core steps): n * q each
         float2* dense_part = nullptr;   // column-chunk partial products of the reduced inverse
@@ -260,6 +263,7 @@ struct ls_handle {
     static constexpr int kLanes = 8;
     SweepLane lanes[kLanes];
     int lane = 0;              // lane the sweep functions use (set around concurrent chunks)
+    int chains = 1;            // chunks running side by side on the lanes (the same)
 
     // Krylov workspaces (FP64): the context of ls_krylov.cu and the staging buffers of
     // the host-array entry points, owned by the handle (no library-global state)

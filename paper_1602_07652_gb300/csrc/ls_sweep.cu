@@ -145,6 +145,7 @@ struct CrStep {
     size_t SB, YB;                 // member strides
     size_t pool_strip, x_strip;    // strip blockIdx.y (elements; the set-up runs all strips at once)
     int nb;
+    bool early;                    // let the successor start at once (one FP32 member, a chain alone)
     bool to_y;                     // MODE 1: the even results go to y (the last level before c)
     const C* inv;                  // MODE 6: S_c^{-1} (nc x nc, column-major), blocks j << c
     int nc, c;
@@ -170,9 +171,9 @@ template <typename T, int MODE, int NB>
 __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(CrStep<T> a) {
     using C = cpx_t<T>;
     constexpr int NM = cr_mats<MODE>(), PF = cr_prefetch<T, MODE>();
-    constexpr bool kEarly = sizeof(T) == 4 && NB == 1;
+    const bool early = sizeof(T) == 4 && NB == 1 && a.early;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (kEarly) pdl_trigger();
+    if (early) pdl_trigger();
     const int q = a.q, ncol = MODE == 6 ? a.nc : q;
     C* vin = reinterpret_cast<C*>(smem_raw);     // [NM][NB][ncol]
     C* red = vin + (size_t)NM * NB * ncol;       // [CG][NB][R]
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(kMvThreads, (cr_min_ctas<T, NB>())) k_cr_step(
     int cend = ncol;
     if (kSparse) cend = __syncthreads_or(nonzero) ? ncol : 0;
     else __syncthreads();
-    if (!kEarly && !(sizeof(T) == 8 && gridDim.x <= 304)) pdl_trigger();   // else at its end
+    if (!early && !(sizeof(T) == 8 && gridDim.x <= 304)) pdl_trigger();   // else at its end
     C part[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) part[b] = czero<C>();
@@ -634,10 +635,19 @@ StripGeom geom_of(const ls_handle* h) { return StripGeom{h->n, h->t, h->E, h->q,
 // product of up to 700 rows, not a block, and is always split: on the three CTAs that its rows
 // need at least, it was the longest step of the solve (unsplit levels, a field of Algorithm 2, ms:
 // 64^2 FP64 2.47 -> 0.52, 400^2 FP64 10.7 -> 6.9, 256^2 FP32 1.80 -> 1.01).
+// Chains that run side by side on the lanes share the SMs, and their CTAs fill them without
+// splitting: the target is divided by the chains, down to about one CTA per SM and level (cr_share),
+// and a step starts its successor only when it has its vectors, so that CTAs that wait do not
+// keep another chain's from their slots.  A field of Algorithm 2 on FP32 steps, 32 fields, ms:
+// chunks of 1 on eight lanes at 256^2 0.29 -> 0.15, 1024^2 2.60 -> 2.22, of 4 0.12 -> 0.065 and
+// 1.12 -> 0.90; FP64, 16 fields in chunks of 1, 128^2 0.43 -> 0.25, 400^2 2.48 -> 2.22.  Two
+// chains keep 304 CTAs (768^2, chunks of 8: 0.576, against 0.606 with 152 and 0.642 with 608).
+constexpr int kCtas = 608;
+int cr_share(const ls_handle* h) { return h->chains >= 4 ? 4 : (h->chains >= 2 ? 2 : 1); }
 template <typename T>
-void cr_split(CrStep<T>& a, int rows, int blocks, int min_rows, bool split) {
-    constexpr int kCtas = 608;
-    int S = split ? kCtas / blocks : 1;
+void cr_split(CrStep<T>& a, int rows, int blocks, int min_rows, int ctas) {
+    int S = ctas / blocks;
+    if (S < 1) S = 1;
     if (S > rows / min_rows) S = rows / min_rows;
     if (S < (rows + kMvThreads - 1) / kMvThreads) S = (rows + kMvThreads - 1) / kMvThreads;   // R <= kMvThreads
     a.R = (rows + S - 1) / S;
@@ -673,6 +683,7 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
     a.SB = SB;
     a.YB = (size_t)n * q;
     a.nb = nb;
+    a.early = h->chains == 1;
     a.src = src;
     a.cp = Couple<T>{static_cast<const C*>(F.cw) + (size_t)l * n * 3 * q,
                      static_cast<const C*>(F.ce) + (size_t)l * n * 3 * q};
@@ -685,7 +696,7 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
         a.nk = lv.nk;
         a.off_a = lv.off_dinv;
         a.to_y = k == a.c - 1;
-        cr_split(a, q, blocks, 8, h->cr_split != 0);
+        cr_split(a, q, blocks, 8, h->cr_split ? kCtas / cr_share(h) : 0);
         a.nlead = lv.neven * a.S;
         return (unsigned)(blocks * a.S);
     };
@@ -697,7 +708,7 @@ int cr_solve_nb(ls_handle* h, int dir, int l, cpx_t<T>* x, size_t SB, int nb, co
         if (k == 1) LS_TRY(ls_launch_pdl(h, k_cr_even<T>, dim3((unsigned)l0.neven, (unsigned)nb), dim3(128), 0, a));
         LS_TRY((cr_launch<T, 1, NB>(h, a, grid)));
     }
-    cr_split(a, a.nc, 1, sizeof(T) == 8 ? 4 : 8, true);
+    cr_split(a, a.nc, 1, sizeof(T) == 8 ? 4 : 8, kCtas);
     LS_TRY((cr_launch<T, 6, NB>(h, a, (unsigned)a.S)));
     for (int k = a.c - 1; k >= 1; --k) {
         if (!F.lev[k].nodd) continue;
@@ -891,11 +902,11 @@ int smem_optin(bool mixed) {
 // demand; the lane's graphs, made for smaller buffers, are dropped).
 static void lane_graphs_free(ls_handle::SweepLane& W) {
     for (int b = 0; b <= kMaxBatch; ++b) {
-        if (W.exec[b]) cudaGraphExecDestroy(W.exec[b]);
-        if (W.graph[b]) cudaGraphDestroy(W.graph[b]);
-        W.exec[b] = nullptr;
-        W.graph[b] = nullptr;
-        W.nodes[b] = 0;
+        for (auto& G : W.graphs[b]) {
+            if (G.exec) cudaGraphExecDestroy(G.exec);
+            if (G.graph) cudaGraphDestroy(G.graph);
+            G = ls_handle::SweepLane::Graph{};
+        }
     }
 }
 
@@ -1071,6 +1082,12 @@ void ls_bd_graph_free(ls_handle* h) {
     for (auto& W : h->lanes) lane_graphs_free(W);
 }
 
+// A graph per share of the chip (the CUDA-core steps' row chunks depend on it).
+static ls_handle::SweepLane::Graph& lane_graph(ls_handle* h, int nb) {
+    const int share = cr_on_tensor_cores<float>(h, nb) ? 0 : cr_share(h) / 2;   // 1, 2, 4 -> 0, 1, 2
+    return h->lanes[h->lane].graphs[nb][share];
+}
+
 // Capture Algorithm 2 for nb right-hand sides on the staging buffers once (the
 // sequence of launches and all pointers are fixed after ls_factor), then replay it.
 static int bd_capture(ls_handle* h, int nb) {
@@ -1105,10 +1122,7 @@ static int bd_capture(ls_handle* h, int nb) {
         cudaGraphDestroy(graph);
         return ls_cuda_fail(e);
     }
-    ls_handle::SweepLane& W = h->lanes[h->lane];
-    W.graph[nb] = graph;
-    W.exec[nb] = exec;
-    W.nodes[nb] = nodes;
+    lane_graph(h, nb) = {graph, exec, nodes};
     return LS_OK;
 }
 
@@ -1120,11 +1134,12 @@ int ls_bd_b(ls_handle* h, const float2* g, float2* v, int nb) {
     LS_TRY(ls_sweep_reserve(h, nb));
     if (!h->opts.use_graphs) return bd_direct_mixed(h, g, v, nb);
     ls_handle::SweepLane& W = h->lanes[h->lane];
-    if (!W.exec[nb]) LS_TRY(bd_capture(h, nb));
+    ls_handle::SweepLane::Graph& G = lane_graph(h, nb);
+    if (!G.exec) LS_TRY(bd_capture(h, nb));
     const size_t N = (size_t)h->n * h->n;
     LS_CUDA(cudaMemcpyAsync(W.bd_in, g, sizeof(float2) * N * nb, cudaMemcpyDeviceToDevice, h->stream));
-    LS_CUDA(cudaGraphLaunch(W.exec[nb], h->stream));
-    h->launches += W.nodes[nb];
+    LS_CUDA(cudaGraphLaunch(G.exec, h->stream));
+    h->launches += G.nodes;
     LS_CUDA(cudaMemcpyAsync(v, W.bd_out, sizeof(float2) * N * nb, cudaMemcpyDeviceToDevice, h->stream));
     return LS_OK;
 }
@@ -1133,6 +1148,7 @@ int ls_bd_b(ls_handle* h, const double2* g, double2* v, int nb) {
     if (nb < 1 || nb > ls_bd_cap(h)) return LS_EINVAL;
     LS_TRY(ls_sweep_reserve(h, nb));
     ls_handle::SweepLane& W = h->lanes[h->lane];
+    ls_handle::SweepLane::Graph& G = lane_graph(h, nb);
     const size_t N = (size_t)h->n * h->n;
     if (h->prec == LS_MIXED) {   // through FP32 copies in the lane's staging buffers
         float2* in = reinterpret_cast<float2*>(W.bd_in);
@@ -1141,18 +1157,18 @@ int ls_bd_b(ls_handle* h, const double2* g, double2* v, int nb) {
         if (!h->opts.use_graphs) {
             LS_TRY(bd_direct_mixed(h, in, out, nb));
         } else {
-            if (!W.exec[nb]) LS_TRY(bd_capture(h, nb));
-            LS_CUDA(cudaGraphLaunch(W.exec[nb], h->stream));
-            h->launches += W.nodes[nb];
+            if (!G.exec) LS_TRY(bd_capture(h, nb));
+            LS_CUDA(cudaGraphLaunch(G.exec, h->stream));
+            h->launches += G.nodes;
         }
         for (int b = 0; b < nb; ++b) LS_TRY(ls_vec_copy(h, out + b * N, v + b * N));
         return LS_OK;
     }
     if (!h->opts.use_graphs) return bd_direct(h, g, v, nb);
-    if (!W.exec[nb]) LS_TRY(bd_capture(h, nb));
+    if (!G.exec) LS_TRY(bd_capture(h, nb));
     LS_CUDA(cudaMemcpyAsync(W.bd_in, g, sizeof(double2) * N * nb, cudaMemcpyDeviceToDevice, h->stream));
-    LS_CUDA(cudaGraphLaunch(W.exec[nb], h->stream));
-    h->launches += W.nodes[nb];
+    LS_CUDA(cudaGraphLaunch(G.exec, h->stream));
+    h->launches += G.nodes;
     LS_CUDA(cudaMemcpyAsync(v, W.bd_out, sizeof(double2) * N * nb, cudaMemcpyDeviceToDevice, h->stream));
     return LS_OK;
 }
@@ -1175,6 +1191,7 @@ static int bd_lanes(ls_handle* h, const FT* g, FT* v, int nb, int chunk, const u
     }
     cudaStream_t main = h->stream;
     LS_CUDA(cudaEventRecord(h->ev_fork, main));
+    h->chains = run.size() < ls_handle::kLanes ? (int)run.size() : ls_handle::kLanes;
     bool used[ls_handle::kLanes] = {};
     int rc = LS_OK;
     for (size_t ci = 0; ci < run.size() && rc == LS_OK; ++ci) {
@@ -1196,6 +1213,7 @@ static int bd_lanes(ls_handle* h, const FT* g, FT* v, int nb, int chunk, const u
         h->stream = main;
         h->lane = 0;
     }
+    h->chains = 1;
     for (int k = 1; k < ls_handle::kLanes; ++k) {  // join, also after a failure
         if (!used[k]) continue;
         cudaEventRecord(h->lanes[k].done, h->lanes[k].stream);

@@ -1,4 +1,13 @@
-"""Forms of the CUDA-core local solves against each other (timed on one handle, best of three)."""
+"""Chunks of a batch side by side: the CUDA-core steps' splitting depends on the number of chains.
+
+A batch's Algorithm 2 runs in chunks on concurrent streams (Sec. 3.5 shared by a batch), and the
+row chunks of the reduction steps are coarser the more chains share the GPU, with a captured
+graph for each form.  Checked: one handle taken through 1, 2, 4 and 8 chains and back solves the
+same fields; a single chain's result keeps its bits after runs of several.  Bound: two solves of
+one problem at tolerance t differ by at most 2 t cond; 1e-7 at t = 1e-10 leaves a factor of 500.
+The two timed tests
+compare forms of one handle with each other, best of three.
+"""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -15,6 +24,33 @@ def _lib():
     binding.load()
 
 
+@pytest.mark.parametrize("graphs", [1, 0])
+@pytest.mark.parametrize("prec,chunks", [(binding.LS_MIXED, (8, 4, 2, 1)), (binding.LS_FP64, (4, 2, 1))])
+@pytest.mark.parametrize("n,L,E", [(72, 2, 6), (111, 3, 10)])
+def test_any_number_of_chains_solves_the_same_fields(n, L, E, prec, chunks, graphs):
+    o = binding.default_opts()
+    o.use_graphs = graphs
+    m = torch.from_numpy(inputs.bump_medium(n, nbumps=4, seed=n)).cuda()
+    s = binding.Solver(m, inputs.omega_for_ppw(n, 10.0), layers=L, ext=E, precision=prec, opts=o)
+    s.ls_factor()
+    if prec == binding.LS_MIXED:
+        s.ls_set_tensor_steps(0)
+    f = torch.stack([s.ls_incident_rhs(0.4 + 0.7 * k) for k in range(8)]).contiguous()
+    top = chunks[0]
+    for split in (1, 0):
+        s.ls_set_reduction(split)
+        alone = s.ls_precond_bd_batch(f[:top].contiguous())
+        ref = None
+        for chunk in chunks + chunks[::-1]:
+            s.ls_set_shapes(4, chunk)
+            u = s.ls_solve_batch(f, 1e-10)[0]
+            ref = u if ref is None else ref
+            err = ((u - ref).abs().square().sum(dim=(1, 2)) / ref.abs().square().sum(dim=(1, 2))).sqrt().max()
+            assert float(err) < 1e-7, (split, chunk, float(err))
+            assert torch.equal(s.ls_precond_bd_batch(f[:top].contiguous()), alone), (split, chunk)
+    s.close()
+
+
 def test_unsplit_levels_do_not_leave_the_reduced_inverse_unsplit():
     # 64^2 in FP64, one field: the forms of the levels differ little at four blocks (1.02 measured);
     # with the inverse's product on three CTAs the unsplit form took 4.8 times the split one's time
@@ -23,4 +59,16 @@ def test_unsplit_levels_do_not_leave_the_reduced_inverse_unsplit():
     s.ls_factor()
     t = min((s.ls_autotune(1, 10) for _ in range(3)), key=lambda d: d["bd_ms_per_rhs_nosplit"][0])
     assert t["bd_ms_per_rhs_nosplit"][0] < 2.5 * t["bd_ms_per_rhs"][0], t
+    s.close()
+
+
+def test_many_chains_do_not_pay_for_splitting():
+    # 256^2, 32 fields, one to a chunk, on eight streams: no row of the table needs splitting then
+    # (split over unsplit 1.03 measured); split as for a chain alone it took 1.9 times the time
+    m = torch.from_numpy(inputs.bump_medium(256, nbumps=4, seed=256)).cuda()
+    s = binding.Solver(m, inputs.omega_for_ppw(256, 10.24), layers=4, ext=10, precision=binding.LS_MIXED)
+    s.ls_factor()
+    s.ls_set_tensor_steps(0)
+    t = min((s.ls_autotune(32, 5) for _ in range(3)), key=lambda d: d["bd_ms_per_rhs"][0])
+    assert t["bd_ms_per_rhs"][0] < 1.5 * t["bd_ms_per_rhs_nosplit"][0], t
     s.close()
