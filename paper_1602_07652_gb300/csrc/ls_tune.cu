@@ -49,6 +49,7 @@ int run_bd(ls_handle* h, void* a) {  // as the batched solve runs it: chunks on 
 extern "C" int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out) {
     if (!h || nrhs < 1 || nrhs > LS_MAX_BATCH || reps < 1) return LS_EINVAL;
     ls_tuning t{};
+    const int user_variant = h->fft_variant, user_split = h->cr_split, user_tc = h->cr_tc;
     const size_t N = (size_t)h->n * h->n;
     double2* buf = nullptr;
     LS_CUDA(cudaMalloc(&buf, sizeof(double2) * N * 2 * nrhs));
@@ -84,7 +85,6 @@ extern "C" int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out) {
         best = 0;
         int chunk = 1, split = 1, tc = 0;
         const int tc_avail = h->tc_ready && h->cr_tc ? 1 : 0;   // switched off by ls_set_tensor_steps: not tried
-        const int tc_user = h->cr_tc;
         for (int form = tc_avail ? 2 : 1; form >= 0 && rc == LS_OK; --form) {  // 2: tensor cores, 1: split, 0: unsplit
             const int want_tc = form == 2, sp = form == 2 ? h->cr_split : form;
             if (h->cr_split != sp || h->cr_tc != 2 * want_tc) {
@@ -109,10 +109,7 @@ extern "C" int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out) {
                 }
             }
         }
-        if (rc != LS_OK) {
-            h->cr_tc = tc_user;
-            break;
-        }
+        if (rc != LS_OK) break;
         if (h->cr_split != split || h->cr_tc != 2 * tc) {
             h->cr_split = split;
             h->cr_tc = 2 * tc;
@@ -125,6 +122,14 @@ extern "C" int ls_autotune(ls_handle* h, int nrhs, int reps, ls_tuning* out) {
     } while (0);
     cudaStreamSynchronize(h->stream);
     cudaFree(buf);
+    if (rc != LS_OK) {   // the handle keeps the choices it came with, not the candidate that failed
+        h->fft_variant = user_variant;
+        if (h->cr_split != user_split || h->cr_tc != user_tc) {
+            h->cr_split = user_split;
+            h->cr_tc = user_tc;
+            ls_bd_graph_free(h);
+        }
+    }
     if (rc == LS_OK && out) *out = t;
     return rc;
 }

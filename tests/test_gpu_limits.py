@@ -1,0 +1,42 @@
+"""Shared-memory limits of the kernels hold for every handle of the process.
+
+The limit (dynamic shared memory beyond 48 KB) belongs to a kernel, not to a handle: whatever
+other handles there are, and whichever thread made them, a handle's calls must launch.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_1602_07652_gb300 import binding, inputs  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_1602_07652_gb300 import build_lib
+    build_lib.build()
+    binding.load()
+
+
+def solver(n, layers, ext, prec=None, **kw):
+    m = torch.from_numpy(inputs.bump_medium(n, nbumps=4, seed=n)).cuda()
+    return binding.Solver(m, inputs.omega_for_ppw(n, 10.0), layers=layers, ext=ext,
+                          precision=binding.LS_MIXED if prec is None else prec, **kw)
+
+
+def test_a_failed_or_finished_autotune_leaves_a_shape_that_works():
+    # n = 1025: P = 4096, whose generic column pass needs 144 KB; n = 520: P = 2048, 72 KB
+    s = solver(1025, 25, 10)
+    u = torch.from_numpy(inputs.random_field(1025, 1).astype(np.complex64)).cuda()
+    ref = s.ls_apply_f32(u)
+    o = solver(520, 10, 10)
+    try:
+        s.ls_autotune(1, 1)
+    except RuntimeError:
+        pass
+    y = s.ls_apply_f32(u)
+    assert float((y - ref).abs().square().sum() / ref.abs().square().sum()) < 1e-10
+    o.close()
+    s.close()
