@@ -459,6 +459,12 @@ FftPlan make_plan(int lp, int lrmax) {
     return p;
 }
 
+// The limit belongs to the kernel, for every handle and thread of the process, so it is always
+// that of the longest transform.  The other generic passes stay below 48 KB: the FP32 row passes
+// at any length, the FP64 and double-float ones because they run at P <= 32 only.
+constexpr int kMaxP = 4096, kMaxPGeneric64 = 32;
+static_assert(row_smem32(kMaxP) <= 48 * 1024 && col_smem(kMaxPGeneric64) <= 48 * 1024 &&
+              row_smem64(kMaxPGeneric64) <= 48 * 1024, "no opt-in");
 template <typename K>
 int allow_smem(K kern, size_t bytes) {
     if (bytes > 48 * 1024) LS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
@@ -491,23 +497,9 @@ int ls_fft_init(ls_handle* h) {
     LS_CUDA(cudaMalloc(&h->inczdf, sizeof(cdfl) * h->n));
     LS_TRY(to_dfl(h, reinterpret_cast<const double*>(h->tw64), reinterpret_cast<dfl*>(h->twdf), 2 * (size_t)P));
     LS_TRY(to_dfl(h, h->m64, h->mdf, N));
-    LS_TRY(allow_smem(k_cols_vec<double, EV, CW64, 0>, col_smem(P)));
-    LS_TRY(allow_smem(k_cols_vec<double, EV, CW64, 1>, col_smem(P)));
-    LS_TRY(allow_smem(k_cols_vec<float, EV, CW32, 0>, col_smem(P)));
-    LS_TRY(allow_smem(k_rows_fwd<double, E64, SrcMU<double, double2>>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_fwd<double, E64, SrcInc<double>>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_fwd<double, E64, SrcGpad>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_inv<double, E64, DstApply<double2>>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_inv<double, E64, DstRhs>, row_smem64(P)));
-    LS_TRY(allow_smem(k_cols_vec<dfl, EV, CW64, 0>, col_smem(P)));
-    LS_TRY(allow_smem(k_rows_fwd<dfl, E64, SrcMU<dfl, double2>>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_fwd<dfl, E64, SrcIncDf>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_inv<dfl, E64, DstApply<double2>>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_inv<dfl, E64, DstRhs>, row_smem64(P)));
-    LS_TRY(allow_smem(k_rows_fwd<float, E32, SrcMU<float, float2>>, row_smem32(P)));
-    LS_TRY(allow_smem(k_rows_fwd<float, E32, SrcMU<float, double2>>, row_smem32(P)));
-    LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<float2>>, row_smem32(P)));
-    LS_TRY(allow_smem(k_rows_inv<float, E32, DstApply<double2>>, row_smem32(P)));
+    LS_TRY(allow_smem(k_cols_vec<double, EV, CW64, 1>, col_smem(kMaxP)));
+    LS_TRY(allow_smem(k_cols_vec<float, EV, CW32, 0>, col_smem(kMaxP)));
+    LS_TRY(allow_smem(k_rows_fwd<double, E64, SrcGpad>, row_smem64(kMaxP)));
     if (h->lp >= 6) {
         LS_CUDA(cudaMalloc(&h->tww64, sizeof(double2) * 2 * P));
         LS_CUDA(cudaMalloc(&h->twwdf, sizeof(cdfl) * 2 * P));
@@ -708,7 +700,7 @@ int noalloc_setup(int dev, cudaStream_t stream, NoAllocDevice** out) {
         d.tw = static_cast<float2*>(p);
         k_noalloc_twiddles<<<(kNoAllocTwElems + 255) / 256, 256, 0, stream>>>(d.tw);
         LS_CUDA(cudaPeekAtLastError());
-        LS_TRY(allow_smem(k_cols_vec<float, EV, CW32, 0>, col_smem(2048)));
+        LS_TRY(allow_smem(k_cols_vec<float, EV, CW32, 0>, col_smem(kMaxP)));
         LS_CUDA(cudaStreamSynchronize(stream));
         d.ready = true;
     }

@@ -40,3 +40,26 @@ def test_a_failed_or_finished_autotune_leaves_a_shape_that_works():
     assert float((y - ref).abs().square().sum() / ref.abs().square().sum()) < 1e-10
     o.close()
     s.close()
+
+
+def test_a_handle_of_a_shorter_transform_leaves_a_longer_one_its_shared_memory():
+    s = solver(1025, 25, 10)
+    u = torch.from_numpy(inputs.random_field(1025, 1).astype(np.complex64)).cuda()
+    ref = s.ls_apply_f32(u)
+    s.ls_set_shapes(1)   # the generic passes
+
+    def check():
+        y = s.ls_apply_f32(u)
+        assert float((y - ref).abs().square().sum() / ref.abs().square().sum()) < 1e-10
+
+    check()
+    k = solver(64, 2, 6)   # the first call without allocation sets a limit of its own
+    g = k.ls_get_spectrum()[0].to(torch.complex64).contiguous()
+    m = torch.zeros((64, 64), dtype=torch.float32, device="cuda")
+    binding.ls_apply_f32_noalloc(64, m, g, torch.zeros((64, 64), dtype=torch.complex64, device="cuda"))
+    check()
+    o = solver(520, 10, 10)
+    check()
+    s.ls_autotune(1, 1)
+    for x in (k, o, s):
+        x.close()
