@@ -100,6 +100,10 @@ __device__ bool gj_invert(double2* M, int q, double2* fcol, int* piv, double* re
     return ok;
 }
 
+constexpr size_t invert_smem(int q) {
+    return ((size_t)q * q + kMaxQ) * sizeof(double2) + 256 * (sizeof(double) + sizeof(int)) + kMaxQ * sizeof(int);
+}
+
 struct InvTask {
     const double2* src;  // dense source (column-major) or null for a level-0 D block
     double2* dst;
@@ -447,8 +451,10 @@ int factor_direction(ls_handle* h, int dir, Scratch& S) {
         LS_CUDA(cudaMalloc(&S.err, sizeof(int)));
     }
     LS_CUDA(cudaMemsetAsync(S.err, 0, sizeof(int), h->stream));
-    const size_t inv_smem = (qq + kMaxQ) * sizeof(double2) + 256 * (sizeof(double) + sizeof(int)) + kMaxQ * sizeof(int);
-    LS_CUDA(cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem));
+    // (the limit is the kernel's, for every handle and thread of the process: that of the tallest
+    // strip, so that no factorisation lowers it under another one's launches)
+    const size_t inv_smem = invert_smem(q);
+    LS_CUDA(cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)invert_smem(kMaxQ)));
     int cur = 0;
     for (int k = 0; k < F.K; ++k) {
         const CrLevel& lv = F.lev[k];

@@ -3,6 +3,8 @@
 The limit (dynamic shared memory beyond 48 KB) belongs to a kernel, not to a handle: whatever
 other handles there are, and whichever thread made them, a handle's calls must launch.
 """
+import threading
+
 import numpy as np
 import pytest
 
@@ -63,3 +65,30 @@ def test_a_handle_of_a_shorter_transform_leaves_a_longer_one_its_shared_memory()
     s.ls_autotune(1, 1)
     for x in (k, o, s):
         x.close()
+
+
+def test_factorisations_of_different_heights_in_several_threads():
+    # q = 112 needs 204 KB a CTA for the inverses, q = 54 needs 51 KB
+    tall = solver(400, 4, 6, binding.LS_FP64, stream=torch.cuda.Stream())
+    short = [solver(50, 1, 2, binding.LS_FP64, stream=torch.cuda.Stream()) for _ in range(4)]
+    torch.cuda.synchronize()
+    errors, done = [], threading.Event()
+
+    def factor(s, more):
+        try:
+            while more():
+                s.ls_factor()
+        except RuntimeError as e:
+            errors.append(e)
+
+    others = [threading.Thread(target=factor, args=(s, lambda: not done.is_set())) for s in short]
+    for t in others:
+        t.start()
+    left = iter(range(10))
+    factor(tall, lambda: next(left, None) is not None)
+    done.set()
+    for t in others:
+        t.join()
+    assert not errors, errors
+    for s in short + [tall]:
+        s.close()
