@@ -92,3 +92,12 @@ def test_factorisations_of_different_heights_in_several_threads():
     assert not errors, errors
     for s in short + [tall]:
         s.close()
+
+
+def test_a_taller_strip_is_factored_after_a_handle_of_a_shorter_one():
+    # the steps that build the reduced inverse ask for 60 KB at q = 112, 50 KB at q = 70
+    tall = solver(200, 2, 6, binding.LS_FP64)
+    short = solver(100, 2, 10, binding.LS_FP64)
+    tall.ls_factor()
+    short.close()
+    tall.close()
