@@ -93,6 +93,13 @@ int ls_cuda_fail(cudaError_t e) {
     return LS_ECUDA;
 }
 
+// A failed allocation's status.  The runtime keeps the error until it is read, and the next launch
+// check (the library's or the caller's) would take it for its own.
+int ls_no_memory() {
+    cudaGetLastError();
+    return LS_ENOMEM;
+}
+
 // Timed intervals are pairs of events recorded on the handle's stream; nothing
 // waits on them until ls_timing_collect, so timing adds no host synchronisation.
 int ls_timing_begin(ls_handle* h) {
@@ -216,16 +223,16 @@ int ls_setup(const ls_grid* grid, double hstep, double omega, const double* m, c
     h->stream = static_cast<cudaStream_t>(stream);
     int rc = LS_OK;
     do {
-        if (cudaGetDevice(&h->device) != cudaSuccess) { rc = LS_ECUDA; break; }
+        if (cudaGetDevice(&h->device) != cudaSuccess) { rc = ls_cuda_fail(cudaGetLastError()); break; }
         const size_t N = (size_t)n * n;
         if (cudaMalloc(&h->m64, sizeof(double) * N) != cudaSuccess ||
             cudaMalloc(&h->m32, sizeof(float) * N) != cudaSuccess ||
             cudaMalloc(&h->mT64, sizeof(double) * N) != cudaSuccess) {
-            rc = LS_ENOMEM;
+            rc = ls_no_memory();
             break;
         }
         if (cudaMemcpyAsync(h->m64, m, sizeof(double) * N, cudaMemcpyDefault, h->stream) != cudaSuccess) {
-            rc = LS_ECUDA;
+            rc = ls_cuda_fail(cudaGetLastError());
             break;
         }
         k_real_to32<<<608, 256, 0, h->stream>>>(N, h->m64, h->m32);
@@ -240,10 +247,10 @@ int ls_setup(const ls_grid* grid, double hstep, double omega, const double* m, c
         if (rc != LS_OK) break;
         if ((rc = ls_sweep_alloc(h)) != LS_OK) break;
         if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess) {
-            rc = LS_ECUDA;
+            rc = ls_cuda_fail(cudaGetLastError());
             break;
         }
-        if (cudaStreamSynchronize(h->stream) != cudaSuccess) { rc = LS_ECUDA; break; }
+        if (cudaStreamSynchronize(h->stream) != cudaSuccess) { rc = ls_cuda_fail(cudaGetLastError()); break; }
     } while (0);
     if (rc != LS_OK) {
         release(h);
@@ -299,15 +306,14 @@ int ls_host_alloc(size_t bytes, void** out) {
     if (bytes == 0) return LS_EINVAL;
     if (cudaHostAlloc(out, bytes, cudaHostAllocPortable) != cudaSuccess) {
         *out = nullptr;
-        cudaGetLastError();   // the failure is reported by the return code
-        return LS_ENOMEM;
+        return ls_no_memory();
     }
     return LS_OK;
 }
 
 int ls_host_free(void* p) {
     if (!p) return LS_OK;
-    return cudaFreeHost(p) == cudaSuccess ? LS_OK : LS_ECUDA;
+    return cudaFreeHost(p) == cudaSuccess ? LS_OK : ls_cuda_fail(cudaGetLastError());
 }
 
 int ls_get_sweep_histogram(ls_handle* h, int* counts, int len) {
@@ -415,7 +421,7 @@ int ls_solve_group(int nprob, ls_handle* const* hs, const ls_c64* const* f, doub
             const int i = next.fetch_add(1);
             if (i >= nprob) return;
             if (cudaSetDevice(hs[i]->device) != cudaSuccess) {
-                rc[i] = LS_ECUDA;
+                rc[i] = ls_cuda_fail(cudaGetLastError());
                 continue;
             }
             rc[i] = ls_solve(hs[i], f[i], tol, u[i], 0, stats ? &stats[i] : nullptr);

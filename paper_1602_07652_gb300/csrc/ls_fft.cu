@@ -533,7 +533,7 @@ int ls_spectrum_build(ls_handle* h, const double2* gtab) {
         k_quad_to32<<<(unsigned)((cnt + 255) / 256), 256, 0, h->stream>>>(cnt, h->ghat64, h->ghat32);
         h->launches++;
         if (cudaMalloc(&h->ghatdf, sizeof(cdfl) * cnt) != cudaSuccess) {
-            rc = LS_ENOMEM;
+            rc = ls_no_memory();
             break;
         }
         if ((rc = to_dfl(h, reinterpret_cast<const double*>(h->ghat64), reinterpret_cast<dfl*>(h->ghatdf),

@@ -317,6 +317,7 @@ struct ls_handle {
     } while (0)
 
 int ls_cuda_fail(cudaError_t e);
+int ls_no_memory();   // LS_ENOMEM, the runtime's own error cleared
 
 // launch + bookkeeping; returns LS_ECUDA from the enclosing function on failure
 #define LS_LAUNCH(hdl, kern, grid, block, smem, ...)                                   \

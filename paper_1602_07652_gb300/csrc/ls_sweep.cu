@@ -963,7 +963,7 @@ int ls_cr_inverse_build(ls_handle* h, int dir) {
     LS_CUDA(cudaMalloc(&A, sizeof(double2) * total));
     int rc = LS_OK;
     do {
-        if (cudaMalloc(&y, sizeof(double2) * total) != cudaSuccess) { rc = LS_ENOMEM; break; }
+        if (cudaMalloc(&y, sizeof(double2) * total) != cudaSuccess) { rc = ls_no_memory(); break; }
         k_identity<<<1216, 256, 0, h->stream>>>(total, nc, A);
         h->launches++;
         CrStep<double> a{};
@@ -1003,7 +1003,7 @@ int ls_cr_inverse_build(ls_handle* h, int dir) {
         }
         if (rc != LS_OK) break;
         if (h->prec == LS_MIXED) {
-            if (cudaMalloc(&F.inv, sizeof(float2) * total) != cudaSuccess) { rc = LS_ENOMEM; break; }
+            if (cudaMalloc(&F.inv, sizeof(float2) * total) != cudaSuccess) { rc = ls_no_memory(); break; }
             k_inverse32<<<1216, 256, 0, h->stream>>>(total, A, static_cast<float2*>(F.inv));
             h->launches++;
         } else {
