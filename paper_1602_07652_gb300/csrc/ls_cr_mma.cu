@@ -441,9 +441,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_cr_mma(StepArgs a) {
             // plane re into accumulator 0 (M_re [X_re | X_im]), plane im into accumulator 1
             const unsigned long long bd0 = sdesc(su32(Bs + (size_t)t * KA * BATOM));
             if (kStages >= 2) {
-                // Both planes of the matrix, slice by slice in turn, so that an MMA (128 x 2NB x 8,
-                // about 145 cycles each whatever NB) does not continue the accumulator of the one
-                // before it: Algorithm 2 of 32 fields 13.4 -> 12.8 ms at 1024^2, 45.2 -> 43.7 at 2048^2.
+                // Both planes of the matrix, slice by slice in turn: Algorithm 2 of 32 fields 13.4 ->
+                // 12.8 ms at 1024^2, 45.2 -> 43.7 at 2048^2.  So little says that the products do not
+                // wait for the accumulator of the one before; what spaces them is not known (the
+                // tensor pipe is 6 to 9 per cent busy over a step).
                 const int s0 = i % kStages, s1 = (i + 1) % kStages;
                 ok = bar_wait(&full[s0], (unsigned)(i / kStages) & 1u) &&
                      bar_wait(&full[s1], (unsigned)((i + 1) / kStages) & 1u);

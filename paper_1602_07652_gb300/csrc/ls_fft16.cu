@@ -1,5 +1,5 @@
 // ls_fft16.cu -- the FP32 LS-apply (Sec. 2) with transforms specialised on the
-// padded length P = 2^LP (256 <= P <= 4096) and on the radix a thread owns.
+// padded length P = 2^LP (32 <= P <= 4096) and on the radix a thread owns.
 //
 // Same three HBM passes as the generic path (rows forward, columns forward x
 // Ghat x inverse, rows inverse), with everything a transform does fixed at
@@ -16,7 +16,7 @@
 //     E/2 inputs (z, x < n <= P/2), so its first butterfly layer only rotates.
 // Radix 16 halves the exchanges, radix 8 halves the registers a thread needs
 // (more resident warps to hide latency); the autotuner picks per problem.
-// Small P groups several transforms per CTA of at least 256 threads.
+// Small P groups several transforms per CTA (of 64 threads; 256 where TMA moves the tiles).
 //
 // The column pass reads and writes 16-byte row segments (2 columns) of the
 // row-major n x P slab, one per row at a stride of 8P bytes.  Through the LSU each
@@ -34,7 +34,9 @@
 // kernels for 32 <= P < 256 and the default tile shapes (ls_fft16_default), back-to-back calls
 // went from 20.5 to 6.3 us (64^2), 21.6 to 8.9 (256^2), 24.6 to 14.9 (512^2), 57.7 to 41.6
 // (1024^2) and 199 to 141 us (2048^2); with the stage-by-stage twiddles and only the outputs
-// that are stored to 8.3 (256^2), 14.0, 37.3 and 123.
+// that are stored to 8.3 (256^2), 14.0, 37.3 and 123.  Part of the step at 2048^2 is the default
+// shape, which tuned handles had before: there an apply went from 149 to 128 us.  A first call on
+// a new field gains less (64^2 1.6 times, 800^2 nothing): its host call and cold caches remain.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

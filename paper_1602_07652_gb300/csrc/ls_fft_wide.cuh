@@ -1,22 +1,23 @@
 // ls_fft_wide.cuh -- the LS-apply's three passes (Sec. 2) for 16-byte complex values: FP64
-// (double2) and double-float (cdfl), specialised on the padded length P = 2^LP.
+// (double2) and double-float (cdp: packed FP32x2 components), specialised on P = 2^LP.
 //
 // Both are bound by arithmetic -- FP64 by its pipe (about 1/64 of the FP32 rate), double-float
-// by FP32 issue slots (a complex add is 22 operations, a product 40) -- so the transforms leave
-// out what a zero-padded convolution does not need: the first forward stage sees only its
-// lower 4 of 8 inputs (x, z < n <= P/2) and the last inverse stage computes only those
-// outputs, a third and a sixth of a stage's additions.  Everything a transform does is fixed
-// at compile time: Stockham stages of radix 8 (the last forward / first inverse stage takes
-// the remaining radix), a thread owning one transform's 8 elements per stage in 32 registers,
-// so that 1024 threads share an SM; every twiddle is a table load.  The generic passes these
-// replace had a run-time plan, 2-column tiles at 128 registers (512 threads an SM) and no
+// by FP32 issue slots (a complex sum is 11 packed instructions, a product 19) -- so the
+// transforms leave out what a zero-padded convolution does not need: the first forward stage
+// sees only its lower 4 of 8 inputs (x, z < n <= P/2) and the last inverse stage computes only
+// those outputs, a third and a sixth of a stage's additions.  Everything a transform does is
+// fixed at compile time: Stockham stages of radix 8 (the last forward / first inverse stage
+// takes the remaining radix), a thread owning one transform's 8 elements per stage in 32
+// registers, so that 1024 threads share an SM (64 registers; the column pass of P = 4096 then
+// spills 172 bytes in double-float and 88 in FP64, the others at most 72); every twiddle is a
+// table load.  The generic passes these replace had a run-time plan, 2-column tiles at 128 registers (512 threads an SM) and no
 // pruning.  One column per transform touches 16 bytes of a row, half a sector; the other half
 // is the next column's and comes from L2, and the passes are far from the memory bound.
 // The passes are launched programmatically, each starting its successor when only its
 // stores are left.
-// Double-float: 2048^2 1129 -> 971 us (FMA pipe 57 per cent busy), 512^2 75 -> 58, 100^2 41 ->
-// 21; FP64: 2048^2 4158 -> 3634 us, 1024^2 917 -> 852 (FP64 pipe 86 per cent busy), 100^2 53
-// -> 34.
+// Double-float: 2048^2 1129 -> 971 us, 512^2 75 -> 58, 100^2 41 -> 21, and 2048^2 -> 759 with
+// packed components and twiddles stage by stage (FMA pipe 60 to 74 per cent busy); FP64: 2048^2
+// 4158 -> 3634 us, 1024^2 917 -> 852 (FP64 pipe 86 per cent busy), 100^2 53 -> 34.
 #pragma once
 
 #include "ls_fft_common.cuh"

@@ -278,7 +278,7 @@ struct ls_handle {
     int learned_steps = 0;
 
     // choices of the autotuner (ls_tune.cu); defaults until ls_autotune runs
-    int fft_variant = 2;       // column-pass shape (ls_fft16_default): radix 16 with 0 = 1-column tiles,
+    int fft_variant = 2;       // column-pass shape (ls_fft_init sets ls_fft16_default's): radix 16 with 0 = 1-column tiles,
                                // 3 CTAs/SM; 2 = 2-column tiles; 3 = 1-column tiles, 2 CTAs/SM; radix 8 with
                                // 4 = 1-column tiles; 5 = 2-column tiles.  1: generic radix-8 4-column tiles
     static constexpr int kFftVariants = 9;

@@ -129,9 +129,9 @@ struct Couple {
 //     each, and the FP64 pipe of those then holds everyone up (a 64^2 FP64 solve: 53 us with
 //     the trigger at once, 41 after the vectors, 36 at the end; at 400^2 145, 144 and 154 us,
 //     so steps of more CTAs keep the second form).
-// A local solve of one right-hand side went from 126.6 to 71 us (768^2, FP32), from 219 to
-// 141 us (400^2, FP64: 27 million multiply-adds, 50 us at the FP64 rate) and from 83 to 36 us
-// (64^2, FP64).
+// A local solve inside Algorithm 2 of one field (gathers and scatters included) went from 124 to
+// 73 us (768^2, FP32), from 219 to 146 us (400^2, FP64: 27 million multiply-adds, 50 us at the
+// FP64 rate) and from 82 to 36 us (64^2, FP64).
 template <typename T>
 struct CrStep {
     using C = cpx_t<T>;
@@ -657,7 +657,9 @@ void cr_split(CrStep<T>& a, int rows, int blocks, int min_rows, int ctas) {
 // Unknowns of the reduced system whose inverse replaces the levels from c on.  Larger means
 // fewer dependent steps and more bytes a solve (nc^2 entries instead of about 2.5 q^2 per
 // block): 8 blocks of 84 rows are one 3.6 MB (FP32) product of 2.5 us instead of seven steps
-// of 2.8 us; 16 blocks would read 14 MB to save two more.
+// of 2.8 us; 16 blocks would read 14 MB to save two more.  For thin strips 700 unknowns are many
+// blocks, and building their inverse shows in ls_factor (512^2 in 512 layers of q = 5, FP64: 0.27
+// -> 1.14 s, 1.0 -> 7.4 GB), which six applications of Algorithm 2 pay back (247 -> 87 ms each).
 constexpr int kInverseMax = 700;
 
 template <typename T, int MODE, int NB>

@@ -1,8 +1,8 @@
 // ls_tune.cu -- a small autotuner for the two shape choices of the on-line path.
 //
-//  * FFT tile shape of the FP32 / mixed LS-apply: radix-16 transforms with
-//    1-column tiles (3 or 2 CTAs per SM) or 2-column tiles (ls_fft16.cu), or
-//    radix-8 transforms on 4-column tiles (generic path of ls_fft.cu);
+//  * FFT tile shape of the FP32 / mixed LS-apply: radix-16 or radix-8 transforms on
+//    1- or 2-column tiles, moved by threads or by TMA (ls_fft16.cu; below P = 256 its
+//    one shape), or radix-8 transforms on 4-column tiles (generic path of ls_fft.cu);
 //  * band-block batching of Algorithm 2: how many right-hand sides share one
 //    pass over the local-solve factors (1, 2, 4 or 8; FP64 up to 4).
 // Each candidate runs once to warm up and is then timed with CUDA events on the
