@@ -45,14 +45,14 @@ def _chained_kernels():
         for k in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\((?:[^()]|\((?:[^()]|\([^()]*\))*\))*\)\s*)?"
                              r"(\w+)\s*\(((?:[^()]|\([^()]*\))*)\)\s*\{", text):
             body = _braced(text, k.end() - 1)
-            if "pdl_wait()" in body:
+            if "pdl_wait()" in body or "griddepcontrol.wait" in body:
                 yield f, k.group(1), k.group(2), body
 
 
 def test_the_chained_kernels_are_found():
     names = {name for _, name, _, _ in _chained_kernels()}
     assert names == {"k_rows16_fwd", "k_cols16", "k_cols16_tma", "k_cols16_tma2", "k_rows16_inv", "k_wide_rows_fwd",
-                     "k_wide_cols", "k_wide_rows_inv", "k_cr_step", "k_cr_even"}
+                     "k_wide_cols", "k_wide_rows_inv", "k_cr_step", "k_cr_even", "k_cr_mma", "k_dense_mma"}
 
 
 def test_chained_kernels_take_only_constants_as_read_only():
