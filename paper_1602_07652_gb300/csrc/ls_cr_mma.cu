@@ -863,7 +863,11 @@ int launch_ka(ls_handle* h, int mode, unsigned grid, const StepArgs& a) {
 static int dense_prepare(ls_handle* h) {
     const int q = h->q, n = h->n;
     const size_t SB = (size_t)n * q;
-    float2* xt = nullptr;
+    struct Scratch {   // freed on every way out
+        float2* p = nullptr;
+        ~Scratch() { cudaFree(p); }
+    } scratch;
+    float2*& xt = scratch.p;
     for (int d = 0; d < 2; ++d) {
         DirFactors& F = h->fac[d];
         cudaFree(F.dense_tc);
@@ -910,7 +914,6 @@ static int dense_prepare(ls_handle* h) {
         F.dense_ks = ks;
     }
     LS_CUDA(cudaStreamSynchronize(h->stream));
-    cudaFree(xt);
     // every lane's buffer of partial products (the lanes run Algorithm 2 chunks concurrently)
     const size_t e = ls_cr_dense_part_elems(h);
     for (auto& W : h->lanes) {

@@ -517,9 +517,9 @@ int ls_spectrum_build(ls_handle* h, const double2* gtab) {
     const FftPlan& pl = h->plan64;
     double2* work = nullptr;
     const size_t q1 = (size_t)(P / 2 + 1);
-    LS_CUDA(cudaMalloc(&work, sizeof(double2) * (size_t)P * P));
-    LS_CUDA(cudaMalloc(&h->ghat64, sizeof(double2) * q1 * q1));
+    LS_CUDA(cudaMalloc(&h->ghat64, sizeof(double2) * q1 * q1));   // (the handle's before the scratch)
     LS_CUDA(cudaMalloc(&h->ghat32, sizeof(float2) * q1 * q1));
+    LS_CUDA(cudaMalloc(&work, sizeof(double2) * (size_t)P * P));
     int rc = LS_OK;
     do {
         SrcGpad src{gtab, n, P};

@@ -1,8 +1,8 @@
 """Failed allocations in set-up and factorisation, on the CPU with a runtime that computes nothing.
 
 Whichever allocation fails, the call reports it, leaves no error behind in the runtime (the next
-launch check, the library's or the caller's, would take it for its own), and the handle can be
-factored again.
+launch check, the library's or the caller's, would take it for its own) and no memory, and the
+handle can be factored again.
 """
 import os
 import shutil
@@ -40,8 +40,10 @@ for k in range(1000):
         fake.fake_fail_at(-1)
         assert lib.ls_factor(h) == 0, (k, "not factored again")
     lib.ls_destroy(h)
+    assert fake.fake_live() == 0, (k, where, fake.fake_live(), "allocations left")
 assert rc == 0 and min(failures.values()) > 10, (rc, failures)
 lib.ls_destroy(h)
+assert fake.fake_live() == 0
 """
 
 
